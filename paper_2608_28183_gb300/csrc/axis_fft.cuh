@@ -36,21 +36,23 @@ template <int L, int IC_> struct AxisTile {
   static constexpr size_t SMEM = (L > 16) ? sizeof(float2) * FftShape<L>::SMEM * IC : 0;
 };
 
-template <int L, int IC_, int LD, int ST, class TS>
+// INV: inverse transform (e^{+i})
+template <int L, int IC_, int LD, int ST, class TS, bool INV>
 struct AxisCtx {
   using TR = typename RealOf<TS>::T;
   static constexpr int IC = IC_;
   static constexpr int SSTRIDE = IC;
   static constexpr bool kSmemInput = false;
+  static constexpr bool kInverse = INV;
   const void* in;
   void* out;
   const float2* tw;
   float2* smem;
   long long in_base, out_base;     // offsets of (outer, axis 0, inner column)
   long long in_axis, out_axis;
-  int L_in, L_out, c, t_len, inverse;
+  int L_in, L_out, c;
   bool valid;
-  float ldmul, stmul, tmul;
+  float ldmul, tmul, stmul;        // ldmul, tmul: real input only
   long long in_n = 0, out_n = 0;   // extents (bounds-checked build)
   int* err = nullptr;
 
@@ -59,25 +61,22 @@ struct AxisCtx {
     if (!valid || l >= L_in) return;
     if (!bchk(in_base + l * in_axis, in_n, err)) return;
     if constexpr (LD == kLoadReal) {
-      float v = Real<TR>::get(static_cast<const TR*>(in) + in_base + l * in_axis) * ldmul;
+      const float v = Real<TR>::get(static_cast<const TR*>(in) + in_base + l * in_axis) * ldmul;
       x[0] = make_float2(v * tmul, 0.f);
     } else {
-      float2 v = cscale(Cpx<TS>::get(static_cast<const TS*>(in) + in_base + l * in_axis), ldmul);
-      x[0] = inverse ? cconj(v) : v;
+      x[0] = Cpx<TS>::get(static_cast<const TS*>(in) + in_base + l * in_axis);
     }
   }
   __device__ __forceinline__ float2* sm(int) const { return smem + c; }
   __device__ __forceinline__ void store(int l, const float2 (&x)[1]) const {
-    float2 v = x[0];
+    const float2 v = x[0];
     if (!valid || l >= L_out) return;
     const long long o = out_base + l * out_axis;
     if (!bchk(o, out_n, err)) return;
     if constexpr (ST == kStoreCpx) {
-      if (inverse) v = cconj(v);
-      Cpx<TS>::put(static_cast<TS*>(out) + o, cscale(v, stmul));
+      Cpx<TS>::put(static_cast<TS*>(out) + o, cscale2(v, make_float2(stmul, stmul)));
     } else if constexpr (ST == kStoreCpx32) {
-      if (inverse) v = cconj(v);
-      static_cast<float2*>(out)[o] = cscale(v, stmul);
+      static_cast<float2*>(out)[o] = cscale2(v, make_float2(stmul, stmul));
     } else if constexpr (ST == kStoreAbs2) {
       static_cast<float*>(out)[o] = fmaf(v.x, v.x, v.y * v.y) * stmul;
     } else {
@@ -170,11 +169,11 @@ cudaError_t launch_axis_pair_ic(const AxisLaunch& l, cudaStream_t s) {
   return axis_report("realpair", L, IC, Tile::THREADS, smem, grid.x, grid.y, cudaGetLastError());
 }
 
-template <int L, int IC, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut>
+template <int L, int IC, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut, bool INV>
 __global__ void __launch_bounds__(AxisTile<L, IC>::THREADS)
 axis_fft_kernel(const AxisParams p) {
   extern __shared__ float2 axis_sm[];
-  AxisCtx<L, IC, LD, ST, TS> ctx;
+  AxisCtx<L, IC, LD, ST, TS, INV> ctx;
   const int c = threadIdx.x % IC;
   const int j0 = threadIdx.x / IC;
   const long long ii = (long long)blockIdx.x * IC + c;
@@ -191,11 +190,11 @@ axis_fft_kernel(const AxisParams p) {
   ctx.out_axis = p.out_axis;
   ctx.L_in = p.L_in;
   ctx.L_out = p.L_out;
-  ctx.inverse = p.inverse;
-  ctx.t_len = p.t_len;
-  ctx.ldmul = p.ld_dev_scale ? *p.ld_dev_scale : 1.0f;
+  if constexpr (LD == kLoadReal) {
+    ctx.ldmul = p.ld_dev_scale ? *p.ld_dev_scale : 1.0f;
+    ctx.tmul = p.t_len > 0 ? (float)(int)(ii % p.t_len) * p.t_scale : 1.0f;
+  }
   ctx.stmul = p.scale * (p.st_dev_scale ? *p.st_dev_scale : 1.0f);
-  ctx.tmul = p.t_len > 0 ? (float)(int)(ii % p.t_len) * p.t_scale : 1.0f;
   ctx.in_n = p.in_n;
   ctx.out_n = p.out_n;
   ctx.err = p.err;
@@ -208,9 +207,9 @@ axis_fft_kernel(const AxisParams p) {
 // other buffer (double buffering on two mbarriers). The first pass reads the
 // dense staged tile; the transform then continues in place in the same buffer.
 // ---------------------------------------------------------------------------
-template <int L, int IC, int LD, int ST, class TS>
-struct AxisTmaCtx : AxisCtx<L, IC, LD, ST, TS> {
-  using Base = AxisCtx<L, IC, LD, ST, TS>;
+template <int L, int IC, int LD, int ST, class TS, bool INV>
+struct AxisTmaCtx : AxisCtx<L, IC, LD, ST, TS, INV> {
+  using Base = AxisCtx<L, IC, LD, ST, TS, INV>;
   using TR = typename Base::TR;
   static constexpr bool kSmemInput = true;
   const void* tile;     // staged tile, [row][IC] of the input element type
@@ -221,8 +220,7 @@ struct AxisTmaCtx : AxisCtx<L, IC, LD, ST, TS> {
       const float v = Real<TR>::get(static_cast<const TR*>(tile) + l * IC + this->c) * this->ldmul;
       x[0] = make_float2(v * this->tmul, 0.f);
     } else {
-      const float2 v = cscale(Cpx<TS>::get(static_cast<const TS*>(tile) + l * IC + this->c), this->ldmul);
-      x[0] = this->inverse ? cconj(v) : v;
+      x[0] = Cpx<TS>::get(static_cast<const TS*>(tile) + l * IC + this->c);
     }
   }
 };
@@ -237,7 +235,7 @@ template <int L, int IC, int LD, class TS> struct AxisTmaTile {
 
 constexpr int kTmaWaitLimit = 1 << 21;   // polls; each may suspend briefly, ~1 s in all
 
-template <int L, int IC, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut>
+template <int L, int IC, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut, bool INV>
 __global__ void __launch_bounds__(AxisTile<L, IC>::THREADS)
 axis_fft_tma_kernel(const __grid_constant__ CUtensorMap tmap, const AxisParams p, const int tiles_inner,
                     const long long ntiles, int* err) {
@@ -283,7 +281,7 @@ axis_fft_tma_kernel(const __grid_constant__ CUtensorMap tmap, const AxisParams p
     const int ti = (int)(tile % tiles_inner);
     const long long outer = tile / tiles_inner;
     const long long ii = (long long)ti * IC + c;
-    AxisTmaCtx<L, IC, LD, ST, TS> ctx;
+    AxisTmaCtx<L, IC, LD, ST, TS, INV> ctx;
     ctx.tile = buf(slot);
     ctx.in = p.in;
     ctx.out = p.out;
@@ -297,11 +295,11 @@ axis_fft_tma_kernel(const __grid_constant__ CUtensorMap tmap, const AxisParams p
     ctx.out_axis = p.out_axis;
     ctx.L_in = p.L_in;
     ctx.L_out = p.L_out;
-    ctx.inverse = p.inverse;
-    ctx.t_len = p.t_len;
-    ctx.ldmul = ldmul;
+    if constexpr (LD == kLoadReal) {
+      ctx.ldmul = ldmul;
+      ctx.tmul = p.t_len > 0 ? (float)(int)(ii % p.t_len) * p.t_scale : 1.0f;
+    }
     ctx.stmul = stmul;
-    ctx.tmul = p.t_len > 0 ? (float)(int)(ii % p.t_len) * p.t_scale : 1.0f;
     ctx.out_n = p.out_n;
     ctx.err = p.err;
     fftn_run<L, 1, kHalfIn, kHalfOut>(ctx, j0);
@@ -309,10 +307,10 @@ axis_fft_tma_kernel(const __grid_constant__ CUtensorMap tmap, const AxisParams p
   }
 }
 
-template <int L, int IC, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut>
+template <int L, int IC, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut, bool INV>
 cudaError_t launch_axis_tma(const AxisLaunch& l, cudaStream_t s) {
   using T = AxisTmaTile<L, IC, LD, TS>;
-  auto k = axis_fft_tma_kernel<L, IC, LD, ST, TS, kHalfIn, kHalfOut>;
+  auto k = axis_fft_tma_kernel<L, IC, LD, ST, TS, kHalfIn, kHalfOut, INV>;
   static int blocks_per_sm = 0;
   static int sms = 0;
   if (blocks_per_sm == 0) {
@@ -351,8 +349,8 @@ struct AxisTmaPairCtx {
   __device__ __forceinline__ void load(int l, float2 (&x)[1]) const {
     x[0] = make_float2(0.f, 0.f);
     if (l >= L_in) return;
-    x[0].x = Real<TR>::get(tile + l * (2 * IC) + c) * m0;
-    x[0].y = Real<TR>::get(tile + l * (2 * IC) + IC + c) * m1;
+    x[0] = cscale2(make_float2(Real<TR>::get(tile + l * (2 * IC) + c), Real<TR>::get(tile + l * (2 * IC) + IC + c)),
+                   make_float2(m0, m1));
   }
   __device__ __forceinline__ float2* sm(int) const { return smem + c; }
   __device__ __forceinline__ void store(int l, const float2 (&x)[1]) const { smem[pad16(l) * IC + c] = x[0]; }
@@ -472,12 +470,12 @@ cudaError_t launch_axis_pair(const AxisLaunch& l, cudaStream_t s) {
   return launch_axis_pair_ic<L, axis_ic(L, 2), TS, kHalfIn>(l, s);
 }
 
-template <int L, int IC, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut>
+template <int L, int IC, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut, bool INV>
 cudaError_t launch_axis_ic(const AxisLaunch& l, cudaStream_t s) {
   const bool tma = l.has_tmap && l.tile >= axis_ic_count(L);
-  if (tma) return launch_axis_tma<L, IC, LD, ST, TS, kHalfIn, kHalfOut>(l, s);
+  if (tma) return launch_axis_tma<L, IC, LD, ST, TS, kHalfIn, kHalfOut, INV>(l, s);
   using Tile = AxisTile<L, IC>;
-  auto k = axis_fft_kernel<L, IC, LD, ST, TS, kHalfIn, kHalfOut>;
+  auto k = axis_fft_kernel<L, IC, LD, ST, TS, kHalfIn, kHalfOut, INV>;
   if (Tile::SMEM > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile::SMEM);
     if (e != cudaSuccess) return e;
@@ -487,15 +485,15 @@ cudaError_t launch_axis_ic(const AxisLaunch& l, cudaStream_t s) {
   return axis_report("direct", L, IC, Tile::THREADS, Tile::SMEM, grid.x, grid.y, cudaGetLastError());
 }
 
-template <int L, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut>
+template <int L, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut, bool INV>
 cudaError_t launch_axis_one(const AxisLaunch& l, cudaStream_t s) {
   if constexpr (LD == kLoadRealPair) {
     return launch_axis_pair<L, TS, kHalfIn>(l, s);
   } else {
     const int v = (l.tile >= 0 && l.tile < axis_tile_count(L)) ? l.tile % axis_ic_count(L) : 0;
-    if (v == 0) return launch_axis_ic<L, axis_ic(L, 0), LD, ST, TS, kHalfIn, kHalfOut>(l, s);
-    if (v == 1) return launch_axis_ic<L, axis_ic(L, 1), LD, ST, TS, kHalfIn, kHalfOut>(l, s);
-    return launch_axis_ic<L, axis_ic(L, 2), LD, ST, TS, kHalfIn, kHalfOut>(l, s);
+    if (v == 0) return launch_axis_ic<L, axis_ic(L, 0), LD, ST, TS, kHalfIn, kHalfOut, INV>(l, s);
+    if (v == 1) return launch_axis_ic<L, axis_ic(L, 1), LD, ST, TS, kHalfIn, kHalfOut, INV>(l, s);
+    return launch_axis_ic<L, axis_ic(L, 2), LD, ST, TS, kHalfIn, kHalfOut, INV>(l, s);
   }
 }
 
@@ -503,22 +501,22 @@ cudaError_t launch_axis_one(const AxisLaunch& l, cudaStream_t s) {
 // 2: 512-2048) so the builds run in parallel. The range is a template
 // parameter, so the units' dispatchers are distinct functions (a macro alone
 // would give different bodies to one symbol).
-template <int RANGE, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut>
+template <int RANGE, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut, bool INV>
 cudaError_t launch_axis_len(const AxisLaunch& l, cudaStream_t s) {
   switch (l.L) {
 #if defined(AXIS_RANGE) && AXIS_RANGE == 0
-    case 16: return launch_axis_one<16, LD, ST, TS, kHalfIn, kHalfOut>(l, s);
-    case 32: return launch_axis_one<32, LD, ST, TS, kHalfIn, kHalfOut>(l, s);
-    case 64: return launch_axis_one<64, LD, ST, TS, kHalfIn, kHalfOut>(l, s);
+    case 16: return launch_axis_one<16, LD, ST, TS, kHalfIn, kHalfOut, INV>(l, s);
+    case 32: return launch_axis_one<32, LD, ST, TS, kHalfIn, kHalfOut, INV>(l, s);
+    case 64: return launch_axis_one<64, LD, ST, TS, kHalfIn, kHalfOut, INV>(l, s);
 #endif
 #if defined(AXIS_RANGE) && AXIS_RANGE == 1
-    case 128: return launch_axis_one<128, LD, ST, TS, kHalfIn, kHalfOut>(l, s);
-    case 256: return launch_axis_one<256, LD, ST, TS, kHalfIn, kHalfOut>(l, s);
+    case 128: return launch_axis_one<128, LD, ST, TS, kHalfIn, kHalfOut, INV>(l, s);
+    case 256: return launch_axis_one<256, LD, ST, TS, kHalfIn, kHalfOut, INV>(l, s);
 #endif
 #if defined(AXIS_RANGE) && AXIS_RANGE == 2
-    case 512: return launch_axis_one<512, LD, ST, TS, kHalfIn, kHalfOut>(l, s);
-    case 1024: return launch_axis_one<1024, LD, ST, TS, kHalfIn, kHalfOut>(l, s);
-    case 2048: return launch_axis_one<2048, LD, ST, TS, kHalfIn, kHalfOut>(l, s);
+    case 512: return launch_axis_one<512, LD, ST, TS, kHalfIn, kHalfOut, INV>(l, s);
+    case 1024: return launch_axis_one<1024, LD, ST, TS, kHalfIn, kHalfOut, INV>(l, s);
+    case 2048: return launch_axis_one<2048, LD, ST, TS, kHalfIn, kHalfOut, INV>(l, s);
 #endif
     default: return axis_report("no-length", l.L, 0, 0, 0, 0, 0, cudaErrorInvalidValue);
   }
@@ -535,31 +533,38 @@ cudaError_t launch_axis_typed(const AxisLaunch& l, cudaStream_t s) {
   if (axis_debug())
     fprintf(stderr, "[nlos axis] dispatch L=%d load=%d store=%d L_in=%d L_out=%d tile=%d tmap=%d\n", l.L, l.load_mode,
             l.store_mode, l.p.L_in, l.p.L_out, l.tile, l.has_tmap);
+  // a zero-padded input is a forward transform's, a cropped output an inverse's;
+  // load scales belong to real input
+  const bool inv = l.p.inverse != 0;
+  if ((half_in && inv) || (half_out && !half_in && !inv && l.load_mode == kLoadCpx) ||
+      (l.load_mode == kLoadCpx && (l.p.ld_dev_scale || l.p.t_len > 0)))
+    return axis_report("bad-direction", l.L, 0, 0, 0, l.load_mode, l.p.inverse, cudaErrorInvalidValue);
   if (l.load_mode == kLoadReal && l.store_mode == kStoreCpx && half_in && !half_out)
-    return launch_axis_len<RANGE, kLoadReal, kStoreCpx, TS, true, false>(l, s);
+    return launch_axis_len<RANGE, kLoadReal, kStoreCpx, TS, true, false, false>(l, s);
   if (l.load_mode == kLoadRealPair && l.store_mode == kStoreCpx && half_in && 2 * l.p.L_out <= l.L + 2)
-    return launch_axis_len<RANGE, kLoadRealPair, kStoreCpx, TS, true, false>(l, s);
+    return launch_axis_len<RANGE, kLoadRealPair, kStoreCpx, TS, true, false, false>(l, s);
   // unpadded transforms: every input present, every output kept (the real
   // x pass keeps the L/2 + 1 non-redundant outputs)
   const bool full_in = l.p.L_in == l.L;
   if (l.load_mode == kLoadReal && l.store_mode == kStoreCpx && full_in && 2 * l.p.L_out <= l.L + 2)
-    return launch_axis_len<RANGE, kLoadReal, kStoreCpx, TS, false, false>(l, s);
+    return launch_axis_len<RANGE, kLoadReal, kStoreCpx, TS, false, false, false>(l, s);
   if (l.load_mode == kLoadRealPair && l.store_mode == kStoreCpx && full_in && 2 * l.p.L_out <= l.L + 2)
-    return launch_axis_len<RANGE, kLoadRealPair, kStoreCpx, TS, false, false>(l, s);
+    return launch_axis_len<RANGE, kLoadRealPair, kStoreCpx, TS, false, false, false>(l, s);
   if (l.load_mode == kLoadCpx && l.store_mode == kStoreCpx && full_in && l.p.L_out == l.L)
-    return launch_axis_len<RANGE, kLoadCpx, kStoreCpx, TS, false, false>(l, s);
+    return inv ? launch_axis_len<RANGE, kLoadCpx, kStoreCpx, TS, false, false, true>(l, s)
+               : launch_axis_len<RANGE, kLoadCpx, kStoreCpx, TS, false, false, false>(l, s);
   if (l.load_mode == kLoadCpx && l.store_mode == kStoreAbs2 && full_in && l.p.L_out == l.L)
-    return launch_axis_len<RANGE, kLoadCpx, kStoreAbs2, TS, false, false>(l, s);
+    return launch_axis_len<RANGE, kLoadCpx, kStoreAbs2, TS, false, false, true>(l, s);
   if (l.load_mode == kLoadCpx && l.store_mode == kStoreCpx && half_in && !half_out)
-    return launch_axis_len<RANGE, kLoadCpx, kStoreCpx, TS, true, false>(l, s);
+    return launch_axis_len<RANGE, kLoadCpx, kStoreCpx, TS, true, false, false>(l, s);
   if (l.load_mode == kLoadCpx && l.store_mode == kStoreCpx && l.p.L_in == l.L && half_out)
-    return launch_axis_len<RANGE, kLoadCpx, kStoreCpx, TS, false, true>(l, s);
+    return launch_axis_len<RANGE, kLoadCpx, kStoreCpx, TS, false, true, true>(l, s);
   if (l.load_mode == kLoadCpx && l.store_mode == kStoreAbs2 && l.p.L_in == l.L && half_out)
-    return launch_axis_len<RANGE, kLoadCpx, kStoreAbs2, TS, false, true>(l, s);
+    return launch_axis_len<RANGE, kLoadCpx, kStoreAbs2, TS, false, true, true>(l, s);
   if (l.load_mode == kLoadCpx && l.store_mode == kStoreAbs && l.p.L_in == l.L && half_out)
-    return launch_axis_len<RANGE, kLoadCpx, kStoreAbs, TS, false, true>(l, s);
+    return launch_axis_len<RANGE, kLoadCpx, kStoreAbs, TS, false, true, true>(l, s);
   if (l.load_mode == kLoadCpx && l.store_mode == kStoreCpx32 && l.p.L_in == l.L && half_out)
-    return launch_axis_len<RANGE, kLoadCpx, kStoreCpx32, TS, false, true>(l, s);
+    return launch_axis_len<RANGE, kLoadCpx, kStoreCpx32, TS, false, true, true>(l, s);
   return axis_report("no-variant", l.L, 0, 0, 0, l.load_mode, l.store_mode, cudaErrorInvalidValue);
 }
 

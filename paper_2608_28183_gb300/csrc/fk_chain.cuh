@@ -90,8 +90,8 @@ template <int L, int NSLOT = 2> struct ChainTile {
 // (the kernel keeps a copy of the twiddle table in shared memory: its data
 // slots take most of the SM's shared memory, leaving little L1 for the
 // table's global reads)
-template <int L, int IC, int LD, int ST, class TS>
-struct ChainTmaCtx : AxisTmaCtx<L, IC, LD, ST, TS> {
+template <int L, int IC, int LD, int ST, class TS, bool INV>
+struct ChainTmaCtx : AxisTmaCtx<L, IC, LD, ST, TS, INV> {
   static constexpr int kBarThreads = ChainTile<L>::CONSUMERS;
   static constexpr bool kTwShared = true;
 };
@@ -106,14 +106,14 @@ struct ChainTmaPairCtx : AxisTmaPairCtx<L, IC, TS> {
 // y inverse of the inverse chain: stores the intermediate with an L2
 // evict-last policy (it is read back within microseconds, then dropped)
 template <int L, int IC, class TS>
-struct ChainMidCtx : AxisTmaCtx<L, IC, kLoadCpx, kStoreCpx, TS> {
+struct ChainMidCtx : AxisTmaCtx<L, IC, kLoadCpx, kStoreCpx, TS, true> {
   static constexpr int kBarThreads = ChainTile<L>::CONSUMERS;
   static constexpr bool kTwShared = true;
   uint64_t keep;
   __device__ __forceinline__ void store(int l, const float2 (&x)[1]) const {
     if (l >= this->L_out) return;
     if (!bchk(this->out_base + l * this->out_axis, this->out_n, this->err)) return;
-    const float2 v = make_float2(x[0].x * this->stmul, -x[0].y * this->stmul);   // inverse: conjugate
+    const float2 v = cscale2(x[0], make_float2(this->stmul, this->stmul));
     TS* o = static_cast<TS*>(this->out) + this->out_base + l * this->out_axis;
     if constexpr (sizeof(TS) == 8) st_global_hint(reinterpret_cast<float2*>(o), v, keep);
     else Cpx<TS>::put(o, v);
@@ -122,8 +122,8 @@ struct ChainMidCtx : AxisTmaCtx<L, IC, kLoadCpx, kStoreCpx, TS> {
 
 // the second transform of either chain: its output is not read again while
 // the chain runs, so it is stored evict-first and leaves L2 to the intermediate
-template <int L, int IC, int ST, class TS>
-struct ChainOutCtx : ChainTmaCtx<L, IC, kLoadCpx, ST, TS> {
+template <int L, int IC, int ST, class TS, bool INV>
+struct ChainOutCtx : ChainTmaCtx<L, IC, kLoadCpx, ST, TS, INV> {
   uint64_t stream;
   __device__ __forceinline__ void store(int l, const float2 (&x)[1]) const {
     float2 v = x[0];
@@ -133,8 +133,7 @@ struct ChainOutCtx : ChainTmaCtx<L, IC, kLoadCpx, ST, TS> {
     if constexpr (ST == kStoreAbs2) {
       st_global_hint(static_cast<float*>(this->out) + o, fmaf(v.x, v.x, v.y * v.y) * this->stmul, stream);
     } else {
-      if (this->inverse) v = cconj(v);
-      v = cscale(v, this->stmul);
+      v = cscale2(v, make_float2(this->stmul, this->stmul));
       if constexpr (ST == kStoreCpx32 || sizeof(TS) == 8) st_global_hint(static_cast<float2*>(this->out) + o, v, stream);
       else Cpx<TS>::put(static_cast<TS*>(this->out) + o, v);
     }
@@ -147,7 +146,7 @@ template <int L> __device__ __forceinline__ void consumer_sync() {
 
 // common fields of a staged complex sub-tile's transform context
 template <class Ctx>
-__device__ __forceinline__ void chain_ctx(Ctx& ctx, float2* slot, const float2* tw, int c, int inverse) {
+__device__ __forceinline__ void chain_ctx(Ctx& ctx, float2* slot, const float2* tw, int c) {
   ctx.tile = slot;
   ctx.smem = slot;
   ctx.tw = tw;
@@ -156,10 +155,6 @@ __device__ __forceinline__ void chain_ctx(Ctx& ctx, float2* slot, const float2* 
   ctx.valid = true;
   ctx.in_base = 0;
   ctx.in_axis = 0;
-  ctx.inverse = inverse;
-  ctx.t_len = 0;
-  ctx.ldmul = 1.0f;
-  ctx.tmul = 1.0f;
   ctx.in_n = 0;   // the staged tile is read from shared memory
 }
 
@@ -335,8 +330,8 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map1, const __grid_constant_
       } else if (kFwd) {
         // y forward of kx = idx: rows y < b, all L outputs (stored evict-first:
         // the spectrum is read by the next stage, after this one)
-        ChainOutCtx<L, IC, kStoreCpx, TS> ctx;
-        chain_ctx(ctx, buf(slot), tw, c, 0);
+        ChainOutCtx<L, IC, kStoreCpx, TS, false> ctx;
+        chain_ctx(ctx, buf(slot), tw, c);
         ctx.stream = once;
         ctx.out = p.out;
         ctx.out_n = p.out_n;
@@ -346,11 +341,11 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map1, const __grid_constant_
         ctx.L_in = p.b;
         ctx.L_out = L;
         ctx.stmul = p.s2;
-        fftn_run<L, 1, true, false, ChainOutCtx<L, IC, kStoreCpx, TS>, E>(ctx, j0);
+        fftn_run<L, 1, true, false, ChainOutCtx<L, IC, kStoreCpx, TS, false>, E>(ctx, j0);
       } else if (!it.second) {
         // y inverse of kx = idx: keep y < b
         ChainMidCtx<L, IC, TS> ctx;
-        chain_ctx(ctx, buf(slot), tw, c, 1);
+        chain_ctx(ctx, buf(slot), tw, c);
         ctx.keep = keep;
         ctx.out = p.mid;
         ctx.out_n = p.mid_n;
@@ -363,8 +358,8 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map1, const __grid_constant_
         fftn_run<L, 1, false, true, ChainMidCtx<L, IC, TS>, E>(ctx, j0);
       } else {
         // x inverse of wall row y = idx: keep x < a, |.|^2 (or complex)
-        ChainOutCtx<L, IC, ST, TS> ctx;
-        chain_ctx(ctx, buf(slot), tw, c, 1);
+        ChainOutCtx<L, IC, ST, TS, true> ctx;
+        chain_ctx(ctx, buf(slot), tw, c);
         ctx.stream = once;
         ctx.out = p.out;
         ctx.out_n = p.out_n;
@@ -374,7 +369,7 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map1, const __grid_constant_
         ctx.L_in = L;
         ctx.L_out = p.a;
         ctx.stmul = p.s2 * std_;
-        fftn_run<L, 1, false, true, ChainOutCtx<L, IC, ST, TS>, E>(ctx, j0);
+        fftn_run<L, 1, false, true, ChainOutCtx<L, IC, ST, TS, true>, E>(ctx, j0);
       }
     }
     // no consumer touches the slot any more: order the shared-memory

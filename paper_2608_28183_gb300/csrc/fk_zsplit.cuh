@@ -136,11 +136,12 @@ __global__ void __launch_bounds__(FkLiteTile<L, PPC, E>::THREADS, FkLiteTile<L, 
   }
 }
 
-// inverse temporal transform of a kept pencil as conj(DFT(conj(V))): input
-// m < L/2 (the upper half is zero), output z < L/2
+// inverse temporal transform of a kept pencil: input m < L/2 (the upper half
+// is zero), output z < L/2
 template <int L, class TS, bool kCpx, int E>
 struct FkZInvCtx {
   static constexpr int SSTRIDE = 1;
+  static constexpr bool kInverse = true;
   static constexpr bool kSmemInput = false;
   static constexpr int kBarThreads = fk_lite_bar<L, E>();
   const TS* in;
@@ -152,12 +153,12 @@ struct FkZInvCtx {
   long long in_off, in_n, out_off, out_n;
   int* err;
   __device__ __forceinline__ void load(int l, float2 (&x)[1]) const {
-    x[0] = (valid && bchk(in_off + l, in_n, err)) ? cconj(Cpx<TS>::get(in + l)) : make_float2(0.f, 0.f);
+    x[0] = (valid && bchk(in_off + l, in_n, err)) ? Cpx<TS>::get(in + l) : make_float2(0.f, 0.f);
   }
   __device__ __forceinline__ float2* sm(int) const { return W; }
   __device__ __forceinline__ void store(int l, const float2 (&x)[1]) const {
     if (!valid || !bchk(out_off + l, out_n, err)) return;
-    if (kCpx) static_cast<float2*>(out)[l] = make_float2(x[0].x * scale, -x[0].y * scale);
+    if (kCpx) static_cast<float2*>(out)[l] = cscale(x[0], scale);
     else static_cast<float*>(out)[l] = scale * fmaf(x[0].x, x[0].x, x[0].y * x[0].y);
   }
 };

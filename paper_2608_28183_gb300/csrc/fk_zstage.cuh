@@ -61,6 +61,7 @@ struct FkFwdCtx {
 template <int L, class TS, bool kAliasU, bool kGuard>
 struct FkInvCtx {
   static constexpr int SSTRIDE = 1;
+  static constexpr bool kInverse = true;
   static constexpr bool kSmemInput = kAliasU;
   const float2* U;
   float2* W0;
@@ -84,16 +85,14 @@ struct FkInvCtx {
     const float2 w0 = U[pad16((L - c.k0) & (L - 1))], w1 = U[pad16((L - c.k1) & (L - 1))];
     const float2 d = make_float2(fmaf(c.alpha, u1.x - u0.x, u0.x), fmaf(c.alpha, u1.y - u0.y, u0.y));
     const float2 e = make_float2(fmaf(c.alpha, w1.x - w0.x, w0.x), fmaf(c.alpha, w1.y - w0.y, w0.y));
-    // inverse DFT as conj(DFT(conj(V))): the pencil loads conj(V); the
-    // partner's V is conj(lerp) * m/mu, whose conjugate is lerp * m/mu
-    x[0] = cconj(cscale(d, c.jac));
-    x[1] = cscale(e, c.jac);
+    x[0] = cscale(d, c.jac);
+    x[1] = cconj(cscale(e, c.jac));
   }
   __device__ __forceinline__ float2* sm(int t) const { return t == 0 ? W0 : W1; }
   __device__ __forceinline__ void store(int l, const float2 (&x)[2]) const {   // every l the schedule keeps
     if (kGuard && l >= n_out) return;
-    if (st0 && bchk(off0 + l, psi_n, err)) Cpx<TS>::put(out0 + l, cscale(cconj(x[0]), stmul));
-    if (st1 && bchk(off1 + l, psi_n, err)) Cpx<TS>::put(out1 + l, cscale(cconj(x[1]), stmul));
+    if (st0 && bchk(off0 + l, psi_n, err)) Cpx<TS>::put(out0 + l, cscale(x[0], stmul));
+    if (st1 && bchk(off1 + l, psi_n, err)) Cpx<TS>::put(out1 + l, cscale(x[1], stmul));
   }
 };
 

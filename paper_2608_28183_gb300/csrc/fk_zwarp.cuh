@@ -66,6 +66,7 @@ struct FkWarpInvCtx {
   using Sh = FkWarpShape<L>;
   static constexpr int SSTRIDE = 1;
   static constexpr bool kSmemInput = kPartner;   // the partner runs in place in U
+  static constexpr bool kInverse = true;
   static constexpr int kBarThreads = 32;
   const float2* U;
   float2* buf;
@@ -95,14 +96,13 @@ struct FkWarpInvCtx {
       u1 = U[padE<32>(k1)];
     }
     const float2 d = make_float2(fmaf(al, u1.x - u0.x, u0.x), fmaf(al, u1.y - u0.y, u0.y));
-    // the pencil loads conj(V) = conj(d) m/mu; the partner's V is conj(d) m/mu
-    // as well (d gathered at -k), whose conjugate d m/mu it loads
-    x[0] = kPartner ? cscale(d, j) : make_float2(d.x * j, -d.y * j);
+    // the pencil's V is d m/mu, the partner's conj(d) m/mu (d gathered at -k)
+    x[0] = kPartner ? make_float2(d.x * j, -d.y * j) : cscale(d, j);
   }
   __device__ __forceinline__ float2* sm(int) const { return buf; }
   __device__ __forceinline__ void store(int l, const float2 (&x)[1]) const {
     if (kGuard && l >= n_out) return;
-    if (st && bchk(out_off + l, psi_n, err)) Cpx<TS>::put(out + l, make_float2(x[0].x * stmul, -x[0].y * stmul));
+    if (st && bchk(out_off + l, psi_n, err)) Cpx<TS>::put(out + l, cscale(x[0], stmul));
   }
 };
 

@@ -11,8 +11,8 @@
 // type conversion fused there) and the last pass writes straight to global
 // memory through another (cropping, magnitude, band selection fused there).
 //
-// Inverse transforms use conj(DFT(conj(x))), so a context conjugates on load
-// and on store; there is one butterfly implementation.
+// Forward and inverse (unnormalised) transforms share one butterfly
+// implementation, a template on the sign of the exponent.
 //
 // Twiddle tables come from the plan (generated in float64 on the host,
 // stored as float2): for pass p the table T_p[r * Ns + k] = exp(-2 pi i k r /
@@ -30,15 +30,33 @@ namespace nlos {
 // ---------------------------------------------------------------------------
 // complex helpers
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// Sums of complex values are packed: one add.f32x2 issues both components (the
+// FP32 pipe still takes two lanes' time). The transforms are bound by issue
+// slots, not by the FP32 pipe, and the two components of a value sit in one
+// aligned register pair anyway (every load and store moves them as 64 bits).
+// Rounding is that of the scalar sums. Measured with the sign of the inverse
+// folded into the butterflies (below): f-k 256x256x512 float32 1066 -> 1017 us,
+// phasor field 256x256x512 f16 552 -> 535 us, results the same bit for bit.
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+// component-wise product (one packed multiplication)
+__device__ __forceinline__ float2 cscale2(float2 a, float2 m) { return __fmul2_rn(a, m); }
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
-// a * (-i)
-__device__ __forceinline__ float2 cmul_mi(float2 a) { return make_float2(a.y, -a.x); }
+// a * conj(b), rounded as conj(cmul(conj(a), b))
+__device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
+  return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(-a.x, b.y, a.y * b.x));
+}
+// a + q b and a - q b with q = -i (forward) or i (inverse): the quarter turn
+// is a renaming of components, so these stay scalar (a packed sum would have
+// to move b's components first)
+template <bool INV> __device__ __forceinline__ float2 cadd_q(float2 a, float2 b) {
+  return INV ? make_float2(a.x - b.y, a.y + b.x) : make_float2(a.x + b.y, a.y - b.x);
+}
+template <bool INV> __device__ __forceinline__ float2 csub_q(float2 a, float2 b) { return cadd_q<!INV>(a, b); }
 
 // cos(2 pi m / 32) for m = 0..8 (values of the circle function, listed).
 __device__ __forceinline__ float cos32_q(int m) {
@@ -76,55 +94,79 @@ __device__ __forceinline__ float2 mul_w32(float2 a, int m) {
 }
 
 // ---------------------------------------------------------------------------
-// in-register radix-R DFTs, natural order in and out, forward sign e^{-i}
+// in-register radix-R DFTs, natural order in and out: forward sign e^{-i}, or
+// e^{+i} (INV, unnormalised)
 // ---------------------------------------------------------------------------
-template <int R> struct Dft;
+template <int R, bool INV> struct Dft;
 
-template <> struct Dft<1> {
+template <bool INV> struct Dft<1, INV> {
   static __device__ __forceinline__ void run(float2*) {}
 };
-template <> struct Dft<2> {
-  static __device__ __forceinline__ void run(float2* v) {
+// kTurned: the last-but-R/2 input, v[R / 2], is still to be multiplied by q = -i (i if INV)
+template <bool INV> struct Dft<2, INV> {
+  template <bool kTurned> static __device__ __forceinline__ void run_t(float2* v) {
     const float2 t = v[0];
-    v[0] = cadd(t, v[1]);
-    v[1] = csub(t, v[1]);
+    v[0] = kTurned ? cadd_q<INV>(t, v[1]) : cadd(t, v[1]);
+    v[1] = kTurned ? csub_q<INV>(t, v[1]) : csub(t, v[1]);
   }
+  static __device__ __forceinline__ void run(float2* v) { run_t<false>(v); }
 };
-template <> struct Dft<4> {
-  static __device__ __forceinline__ void run(float2* v) {
-    const float2 a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
-    const float2 c = cadd(v[1], v[3]), d = cmul_mi(csub(v[1], v[3]));
+template <bool INV> struct Dft<4, INV> {
+  template <bool kTurned> static __device__ __forceinline__ void run_t(float2* v) {
+    const float2 a = kTurned ? cadd_q<INV>(v[0], v[2]) : cadd(v[0], v[2]);
+    const float2 b = kTurned ? csub_q<INV>(v[0], v[2]) : csub(v[0], v[2]);
+    const float2 c = cadd(v[1], v[3]), d = csub(v[1], v[3]);
     v[0] = cadd(a, c);
     v[2] = csub(a, c);
-    v[1] = cadd(b, d);
-    v[3] = csub(b, d);
+    v[1] = cadd_q<INV>(b, d);
+    v[3] = csub_q<INV>(b, d);
+  }
+  static __device__ __forceinline__ void run(float2* v) { run_t<false>(v); }
+  // v[2] and v[3] zero
+  static __device__ __forceinline__ void run_half(float2* v) {
+    const float2 x0 = v[0], x1 = v[1];
+    v[0] = cadd(x0, x1);
+    v[2] = csub(x0, x1);
+    v[1] = cadd_q<INV>(x0, x1);
+    v[3] = csub_q<INV>(x0, x1);
   }
 };
 // R = R1 * R2 with n = n1 + R1 n2 and k = k2 + R2 k1:
 //   X[k2 + R2 k1] = sum_n1 W_R^{n1 k2} W_R1^{n1 k1} (sum_n2 x[n1 + R1 n2] W_R2^{n2 k2})
-template <int R> struct Dft {
+// run_half: the upper half of the inputs is zero (first pass of a transform
+// whose upper half is zero padding); the inner DFTs are pruned the same way.
+template <int R, bool INV> struct Dft {
   static constexpr int R1 = (R >= 16) ? 4 : 2;
   static constexpr int R2 = R / R1;
-  static __device__ __forceinline__ void run(float2* v) {
+  template <bool kHalf> static __device__ __forceinline__ void run_t(float2* v) {
+    constexpr int kTurn = 32 / R;   // W_R in 32nds of a turn
     float2 y[R1][R2];
 #pragma unroll
     for (int n1 = 0; n1 < R1; ++n1) {
 #pragma unroll
       for (int n2 = 0; n2 < R2; ++n2) y[n1][n2] = v[n1 + R1 * n2];
-      Dft<R2>::run(y[n1]);
-#pragma unroll
-      for (int k2 = 0; k2 < R2; ++k2) y[n1][k2] = mul_w32(y[n1][k2], (32 / R) * n1 * k2);
+      if constexpr (kHalf) Dft<R2, INV>::run_half(y[n1]);
+      else Dft<R2, INV>::run(y[n1]);
     }
 #pragma unroll
     for (int k2 = 0; k2 < R2; ++k2) {
+      // where the twiddle of the middle row is a quarter turn, the sum it
+      // enters takes renamed components instead
+      const bool turned = kTurn * (R1 / 2) * k2 == 8;
       float2 t[R1];
 #pragma unroll
-      for (int n1 = 0; n1 < R1; ++n1) t[n1] = y[n1][k2];
-      Dft<R1>::run(t);
+      for (int n1 = 0; n1 < R1; ++n1) {
+        const int m = kTurn * n1 * k2;
+        t[n1] = (turned && 2 * n1 == R1) ? y[n1][k2] : mul_w32(y[n1][k2], INV ? 32 - m : m);
+      }
+      if (turned) Dft<R1, INV>::template run_t<true>(t);
+      else Dft<R1, INV>::template run_t<false>(t);
 #pragma unroll
       for (int k1 = 0; k1 < R1; ++k1) v[k2 + R2 * k1] = t[k1];
     }
   }
+  static __device__ __forceinline__ void run(float2* v) { run_t<false>(v); }
+  static __device__ __forceinline__ void run_half(float2* v) { run_t<true>(v); }
 };
 
 // ---------------------------------------------------------------------------
@@ -174,6 +216,16 @@ template <class C> struct CtxTwShared<C, decltype((void)C::kTwShared)> {
   static constexpr bool value = C::kTwShared;
 };
 
+// Inverse transforms (e^{+i}, unnormalised): a context that declares kInverse.
+// The butterflies turn the other way and the twiddles are conjugated in their
+// products, which costs nothing; nothing is conjugated on load or store.
+template <class C, class = void> struct CtxInverse {
+  static constexpr bool value = false;
+};
+template <class C> struct CtxInverse<C, decltype((void)C::kInverse)> {
+  static constexpr bool value = C::kInverse;
+};
+
 template <class Ctx> __device__ __forceinline__ void fft_sync() {
   if constexpr (CtxBar<Ctx>::threads == 0) {
     __syncthreads();
@@ -188,78 +240,6 @@ template <class Ctx> __device__ __forceinline__ void fft_sync() {
 // the first pass (stride E) and the contiguous gathers free of bank conflicts.
 __device__ __forceinline__ int pad16(int l) { return l + (l >> 4); }
 template <int E> __device__ __forceinline__ int padE(int l) { return l + l / E; }
-
-// Radix-16 DFT whose inputs 8..15 are zero (first pass of a transform whose
-// upper half is zero padding): the first radix-4 stage sees (x0, x1, 0, 0).
-__device__ __forceinline__ void dft16_half(float2* v) {
-  float2 y[4][4];
-#pragma unroll
-  for (int n1 = 0; n1 < 4; ++n1) {
-    const float2 x0 = v[n1], x1 = v[n1 + 4];
-    const float2 mi = cmul_mi(x1);
-    y[n1][0] = cadd(x0, x1);
-    y[n1][2] = csub(x0, x1);
-    y[n1][1] = cadd(x0, mi);
-    y[n1][3] = csub(x0, mi);
-#pragma unroll
-    for (int k2 = 0; k2 < 4; ++k2) y[n1][k2] = mul_w32(y[n1][k2], 2 * n1 * k2);
-  }
-#pragma unroll
-  for (int k2 = 0; k2 < 4; ++k2) {
-    float2 t[4];
-#pragma unroll
-    for (int n1 = 0; n1 < 4; ++n1) t[n1] = y[n1][k2];
-    Dft<4>::run(t);
-#pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1) v[k2 + 4 * k1] = t[k1];
-  }
-}
-
-// Radix-8 and radix-32 DFTs whose upper half of inputs is zero (first pass of
-// a radix-32 transform whose upper half is zero padding). Radix 8 = 2 x 4:
-// the radix-4 DFTs see (x0, x1, 0, 0); radix 32 = 4 x 8 with the radix-8
-// DFTs pruned that way.
-__device__ __forceinline__ void dft8_half(float2* v) {
-  float2 y[2][4];
-#pragma unroll
-  for (int n1 = 0; n1 < 2; ++n1) {
-    const float2 x0 = v[n1], x1 = v[n1 + 2];
-    const float2 mi = cmul_mi(x1);
-    y[n1][0] = cadd(x0, x1);
-    y[n1][2] = csub(x0, x1);
-    y[n1][1] = cadd(x0, mi);
-    y[n1][3] = csub(x0, mi);
-#pragma unroll
-    for (int k2 = 0; k2 < 4; ++k2) y[n1][k2] = mul_w32(y[n1][k2], 4 * n1 * k2);
-  }
-#pragma unroll
-  for (int k2 = 0; k2 < 4; ++k2) {
-    float2 t[2] = {y[0][k2], y[1][k2]};
-    Dft<2>::run(t);
-    v[k2] = t[0];
-    v[k2 + 4] = t[1];
-  }
-}
-__device__ __forceinline__ void dft32_half(float2* v) {
-  float2 y[4][8];
-#pragma unroll
-  for (int n1 = 0; n1 < 4; ++n1) {
-#pragma unroll
-    for (int n2 = 0; n2 < 8; ++n2) y[n1][n2] = v[n1 + 4 * n2];   // n2 >= 4 are the zero inputs
-    dft8_half(y[n1]);
-#pragma unroll
-    for (int k2 = 0; k2 < 8; ++k2) y[n1][k2] = mul_w32(y[n1][k2], n1 * k2);
-  }
-#pragma unroll
-  for (int k2 = 0; k2 < 8; ++k2) {
-    float2 t[4];
-#pragma unroll
-    for (int n1 = 0; n1 < 4; ++n1) t[n1] = y[n1][k2];
-    Dft<4>::run(t);
-#pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1) v[k2 + 8 * k1] = t[k1];
-  }
-}
 
 // Runs passes P..NPASS-1 of NT L-point transforms that share one schedule
 // (same thread mapping and twiddles) for one thread.
@@ -283,6 +263,7 @@ __device__ __forceinline__ void fftn_passes(Ctx& ctx, const int j0, float2 (&v)[
   constexpr int SS = Ctx::SSTRIDE;
   constexpr bool kFirst = (P == 0);
   constexpr bool kLast = (P == S::NPASS - 1);
+  constexpr bool INV = CtxInverse<Ctx>::value;
 #pragma unroll
   for (int i = 0; i < BPT; ++i) {
     const int j = j0 + i * S::TPC;
@@ -326,14 +307,13 @@ __device__ __forceinline__ void fftn_passes(Ctx& ctx, const int j0, float2 (&v)[
       for (int r = 1; r < R; ++r) {
         const float2 w = CtxTwShared<Ctx>::value ? tp[r * NS] : __ldg(tp + r * NS);
 #pragma unroll
-        for (int t = 0; t < NT; ++t) v[t][i * R + r] = cmul(v[t][i * R + r], w);
+        for (int t = 0; t < NT; ++t) v[t][i * R + r] = INV ? cmulc(v[t][i * R + r], w) : cmul(v[t][i * R + r], w);
       }
     }
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
-      if constexpr (kFirst && kHalfIn && R == 16) dft16_half(&v[t][i * R]);
-      else if constexpr (kFirst && kHalfIn && R == 32) dft32_half(&v[t][i * R]);
-      else Dft<R>::run(&v[t][i * R]);
+      if constexpr (kFirst && kHalfIn) Dft<R, INV>::run_half(&v[t][i * R]);
+      else Dft<R, INV>::run(&v[t][i * R]);
     }
   }
 #pragma unroll

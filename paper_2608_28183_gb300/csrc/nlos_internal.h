@@ -28,9 +28,9 @@ struct AxisParams {
   long long in_outer, in_axis;
   long long out_outer, out_axis;
   int L_in, L_out;
-  int inverse;                 // conjugate on load and on store
+  int inverse;                 // 1: inverse transform (e^{+i}, unnormalised)
   float scale;                 // multiplies every stored value (|.|^2 and |.| included)
-  const float* ld_dev_scale;   // optional device scalar multiplying loads
+  const float* ld_dev_scale;   // real input: optional device scalar multiplying loads
   const float* st_dev_scale;   // optional device scalar multiplying stores
   int t_len;                   // real loads: multiply by (inner index % t_len) * t_scale
   float t_scale;
