@@ -19,8 +19,16 @@
 //
 // The intermediate of a chunk (about 8 MB at 256 x 256) is read within a few
 // microseconds of being written; once its TMA copies have landed, its L2
-// lines are dropped without write-back (discard.global.L2; float32 storage,
-// where a chunk row is one 128-byte line), so it never reaches DRAM.
+// lines are dropped without write-back (discard.global.L2), so it never
+// reaches DRAM.
+//
+// The inverse's input and both intermediates are blocked by 8 columns
+// (nlos_internal.h), so a sub-tile is one contiguous run of memory and one bulk
+// copy. Row by row, as tiled TMA boxes of 8 columns (64-byte rows, 32 bytes
+// in 16-bit storage), the copies cost about 3.5 cycles a row and SM and
+// bounded the inverse: with the transforms and stores left out its copies
+// alone took 295 us of 393 at 256x256x512 float32, and 260 of 428 in f16.
+// The writers pay with 64-byte (32-byte) segments, which L2 merges.
 #pragma once
 #include "axis_fft.cuh"
 #include "nlos_bounds.cuh"
@@ -109,11 +117,20 @@ template <int L, int IC, class TS>
 struct ChainMidCtx : AxisTmaCtx<L, IC, kLoadCpx, kStoreCpx, TS, true> {
   static constexpr int kBarThreads = ChainTile<L>::CONSUMERS;
   static constexpr bool kTwShared = true;
+  static constexpr bool kLoadRow = sizeof(TS) == 8;   // places in psi_pos order
   uint64_t keep;
+  // ky = j + r Q lies at place psi_pos(ky, L / 2) of the tile: rows r and
+  // r + R / 2 share pairs of places (Q is even, so ky's parity is j's)
+  __device__ __forceinline__ void load_row(int j, int r, int Q, int R, float2 (&x)[1]) const {
+    const int h = R / 2;
+    const int place = 2 * (j + (r < h ? r : r - h) * Q) + ((r < h ? 0 : 1) ^ (j & 1));
+    x[0] = Cpx<TS>::get(static_cast<const TS*>(this->tile) + place * IC + this->c);
+  }
   __device__ __forceinline__ void store(int l, const float2 (&x)[1]) const {
     if (l >= this->L_out) return;
     if (!bchk(this->out_base + l * this->out_axis, this->out_n, this->err)) return;
-    const float2 v = cscale2(x[0], make_float2(this->stmul, this->stmul));
+    // (float32 passes carry no scale)
+    const float2 v = sizeof(TS) == 8 ? x[0] : cscale2(x[0], make_float2(this->stmul, this->stmul));
     TS* o = static_cast<TS*>(this->out) + this->out_base + l * this->out_axis;
     if constexpr (sizeof(TS) == 8) st_global_hint(reinterpret_cast<float2*>(o), v, keep);
     else Cpx<TS>::put(o, v);
@@ -133,7 +150,7 @@ struct ChainOutCtx : ChainTmaCtx<L, IC, kLoadCpx, ST, TS, INV> {
     if constexpr (ST == kStoreAbs2) {
       st_global_hint(static_cast<float*>(this->out) + o, fmaf(v.x, v.x, v.y * v.y) * this->stmul, stream);
     } else {
-      v = cscale2(v, make_float2(this->stmul, this->stmul));
+      if constexpr (ST == kStoreCpx32 || sizeof(TS) != 8) v = cscale2(v, make_float2(this->stmul, this->stmul));
       if constexpr (ST == kStoreCpx32 || sizeof(TS) == 8) st_global_hint(static_cast<float2*>(this->out) + o, v, stream);
       else Cpx<TS>::put(static_cast<TS*>(this->out) + o, v);
     }
@@ -163,7 +180,7 @@ __device__ __forceinline__ void chain_ctx(Ctx& ctx, float2* slot, const float2* 
 // complex transform) and n2 = L/2 + 1 y items (one kx, two sub-tiles of 8
 // complex columns); inverse n1 = L y items (one kx) and n2 = b x items (one
 // y), two sub-tiles each.
-// map1 / map2: tensor maps of the first / second transform's input.
+// map: tensor map of the transient (forward).
 //
 // Warp roles: warps 0 .. CONSUMERS/32 - 1 transform sub-tiles; the last warp
 // (one elected lane) takes tickets, waits for chunk counters and issues the
@@ -176,8 +193,7 @@ __device__ __forceinline__ void chain_ctx(Ctx& ctx, float2* slot, const float2* 
 // consumers: the kernel cannot deadlock, and every wait is bounded.
 template <int L, class TS, bool kFwd, int ST, int NSLOT>
 __global__ void __launch_bounds__(ChainTile<L, NSLOT>::THREADS, ChainTile<L, NSLOT>::MIN_BLOCKS)
-fk_chain_kernel(const __grid_constant__ CUtensorMap map1, const __grid_constant__ CUtensorMap map2,
-                const FkChainParams p) {
+fk_chain_kernel(const __grid_constant__ CUtensorMap map, const FkChainParams p) {
   using T = ChainTile<L, NSLOT>;
   using TR = typename RealOf<TS>::T;
   constexpr int IC = kChainIC;
@@ -194,6 +210,10 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map1, const __grid_constant_
   const int n2 = kFwd ? hx : p.b;
   const int total = p.nchunks * (n1 + n2);
   const long long bn = (long long)p.b * p.n;
+  const TS* mid_in = static_cast<const TS*>(p.mid);
+  // second-transform sub-tiles of the intermediate: runs of mid_run elements,
+  // run (block, idx) at (block * n2 + idx) * mid_run
+  const int mid_run = (kFwd ? p.b : L) * IC;
   int* done = p.sync + 1;
   auto subs_of = [&](const ChainItem& it) { return (kFwd && !it.second) ? 1 : 2; };
 
@@ -211,7 +231,7 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map1, const __grid_constant_
     // ------------------------------ producer ------------------------------
     if (threadIdx.x != T::CONSUMERS) return;
     // the inverse's input spectrum is read once: keep L2 for the intermediate
-    const uint64_t once = l2_policy_evict_first();
+    const uint64_t once = l2_policy_evict_first(), keep = l2_policy_evict_last();
     int t = -1, sub = 0;
     for (int k = 0;; ++k) {
       const int slot = k % NSLOT;
@@ -253,18 +273,22 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map1, const __grid_constant_
         fence_proxy_async_global();
       }
       d.state = 0;
-      const bool xreal = kFwd && !it.second;
-      const int rows = kFwd ? (it.second ? p.b : p.a) : L;
-      const size_t row_bytes = (size_t)IC * (xreal ? 2 * sizeof(TR) : sizeof(TS));
-      mbar_arrive_expect_tx(&full[slot], (uint32_t)(rows * row_bytes));
-      for (int r0 = 0; r0 < rows; r0 += 256) {
-        unsigned char* dst = reinterpret_cast<unsigned char*>(buf(slot)) + (size_t)r0 * row_bytes;
-        if (xreal)
-          tma_load_3d(dst, &map1, &full[slot], it.idx * p.n + it.chunk * kChainCols, r0, 0);
-        else if (it.second)
-          tma_load_3d(dst, &map2, &full[slot], it.chunk * kChainCols + sub * IC, r0, it.idx);
-        else
-          tma_load_3d_hint(dst, &map1, &full[slot], it.chunk * kChainCols + sub * IC, r0, it.idx, once);
+      const long long block = 2LL * it.chunk + sub;
+      if (it.second) {
+        const uint32_t bytes = (uint32_t)(mid_run * sizeof(TS));
+        mbar_arrive_expect_tx(&full[slot], bytes);
+        bulk_load_hint(buf(slot), mid_in + (block * n2 + it.idx) * mid_run, bytes, &full[slot], keep);
+      } else if (kFwd) {
+        const size_t row_bytes = (size_t)kChainCols * sizeof(TR);
+        mbar_arrive_expect_tx(&full[slot], (uint32_t)(p.a * row_bytes));
+        for (int r0 = 0; r0 < p.a; r0 += 256)
+          tma_load_3d(reinterpret_cast<unsigned char*>(buf(slot)) + (size_t)r0 * row_bytes, &map, &full[slot],
+                      it.idx * p.n + it.chunk * kChainCols, r0, 0);
+      } else {
+        const uint32_t bytes = (uint32_t)(L * IC * sizeof(TS));
+        mbar_arrive_expect_tx(&full[slot], bytes);
+        bulk_load_hint(buf(slot), static_cast<const TS*>(p.in) + ((long long)it.idx * (p.n / IC) + block) * (L * IC), bytes,
+                       &full[slot], once);
       }
     }
   }
@@ -288,16 +312,16 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map1, const __grid_constant_
     const int nsubs = subs_of(it);
     if (d.state == 0) {
       const int col0 = it.chunk * kChainCols + d.sub * IC;
-      // drop the consumed intermediate from L2: both sub-tiles of this
-      // second-transform item have landed
-      if (p.discard && it.second && d.sub == nsubs - 1) {
-        const int nl = kFwd ? p.b : L;
-        const float2* base = static_cast<const float2*>(p.mid) + (long long)it.chunk * kChainCols;
-        for (int r = threadIdx.x; r < nl; r += T::CONSUMERS) {
-          const long long o = (long long)it.chunk * kChainCols +
-                              (kFwd ? (long long)it.idx * bn + (long long)r * p.n : (long long)r * bn + (long long)it.idx * p.n);
-          if (bchk(o + kChainCols - 1, p.mid_n, p.err)) l2_discard(base + (o - (long long)it.chunk * kChainCols));
-        }
+      const long long block = 2LL * it.chunk + d.sub;
+      // drop the consumed sub-tile of the intermediate from L2: the 128-byte
+      // lines that lie wholly in its run (the run's ends may share a line
+      // with the neighbouring items' runs)
+      if (p.discard && it.second) {
+        constexpr int kLine = 128 / (int)sizeof(TS);
+        const long long o0 = (block * n2 + it.idx) * mid_run;
+        for (long long o = (o0 + kLine - 1) / kLine * kLine + (long long)threadIdx.x * kLine; o + kLine <= o0 + mid_run;
+             o += (long long)T::CONSUMERS * kLine)
+          if (bchk(o + kLine - 1, p.mid_n, p.err)) l2_discard(mid_in + o);
       }
       if (kFwd && !it.second) {
         // x forward of wall row y = idx: 16 real columns t0 + c, t0 + c + 8
@@ -316,15 +340,17 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map1, const __grid_constant_
         // X_{c+8}[k] = (Z[k] - conj Z[L-k]) / (2i), k in [0, L/2]
         const float h = 0.5f * p.s1;
         const float2* z = buf(slot);
-        const long long oo = (long long)it.idx * p.n + t0 + c;
+        const int row = p.b * IC;                            // elements per (block, kx)
+        const long long oo = block * hx * row + it.idx * IC + c;   // block = 2 chunk: columns t0 .. t0 + 7
+        const long long next = (long long)hx * row;          // the block of columns t0 + 8 ..
         TS* o0 = static_cast<TS*>(p.mid) + oo;
         for (int q = j0; q < hx; q += TPC) {
           const float2 zk = z[padE<E>(q) * IC + c];
           const float2 zm = z[padE<E>((L - q) & (L - 1)) * IC + c];
-          TS* o = o0 + q * bn;
-          if (bchk(oo + q * bn + IC, p.mid_n, p.err)) {
+          TS* o = o0 + q * row;
+          if (bchk(oo + q * row + next, p.mid_n, p.err)) {
             Cpx<TS>::put(o, make_float2((zk.x + zm.x) * h, (zk.y - zm.y) * h));
-            Cpx<TS>::put(o + IC, make_float2((zk.y + zm.y) * h, (zm.x - zk.x) * h));
+            Cpx<TS>::put(o + next, make_float2((zk.y + zm.y) * h, (zm.x - zk.x) * h));
           }
         }
       } else if (kFwd) {
@@ -350,8 +376,8 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map1, const __grid_constant_
         ctx.out = p.mid;
         ctx.out_n = p.mid_n;
         ctx.err = p.err;
-        ctx.out_base = (long long)it.idx * bn + col0 + c;
-        ctx.out_axis = p.n;
+        ctx.out_base = (block * p.b * L + it.idx) * IC + c;
+        ctx.out_axis = L * IC;
         ctx.L_in = L;
         ctx.L_out = p.b;
         ctx.stmul = p.s1;
@@ -391,7 +417,7 @@ template <int L, class TS, int NSLOT>
 cudaError_t launch_fk_chain_one(const FkChainLaunch& l, cudaStream_t s) {
   using T = ChainTile<L, NSLOT>;
   const FkChainParams& p = l.p;
-  void (*k)(const __grid_constant__ CUtensorMap, const __grid_constant__ CUtensorMap, const FkChainParams) =
+  void (*k)(const __grid_constant__ CUtensorMap, const FkChainParams) =
       l.fwd ? fk_chain_kernel<L, TS, true, kStoreCpx, NSLOT>
             : l.store_mode == kStoreCpx32 ? fk_chain_kernel<L, TS, false, kStoreCpx32, NSLOT>
             : l.store_mode == kStoreCpx   ? fk_chain_kernel<L, TS, false, kStoreCpx, NSLOT>
@@ -417,7 +443,7 @@ cudaError_t launch_fk_chain_one(const FkChainLaunch& l, cudaStream_t s) {
   FkChainParams q = p;
   q.lag = 1 + (grid + per_chunk - 1) / per_chunk;
   if (q.lag > q.nchunks) q.lag = q.nchunks;
-  k<<<grid, T::THREADS, T::SMEM, s>>>(l.map1, l.map2, q);
+  k<<<grid, T::THREADS, T::SMEM, s>>>(l.map, q);
   return cudaGetLastError();
 }
 

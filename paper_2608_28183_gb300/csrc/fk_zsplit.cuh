@@ -10,8 +10,8 @@
 //       the resampled spectra of the pencil and of its Hermitian partner,
 //       V(m) = lerp(U at the Stolt source) * m / mu for 1 <= m < L/2 and its
 //       partner's conj(lerp(U at minus the source)) * m / mu, both written to
-//       global memory as they are ([kx][ky][m], m < n = L/2; V = 0 for m <= 0
-//       and above L/2);
+//       global memory as they are (m < n = L/2; V = 0 for m <= 0 and above
+//       L/2), blocked by 8 columns for the lateral inverse (FkZParams);
 //   FK4: the lateral inverses (y then x, crop) of V, complex (the fused pair
 //       of fk_chain.cuh);
 //   FK5 (fk_zinv_kernel): per kept pencil (x, y) the inverse temporal
@@ -79,43 +79,91 @@ template <int L, int PPC, int E> struct FkLiteTile {
   static constexpr int MINB = (E == 32 && L == 1024 && THREADS * 80 <= 65536) ? 65536 / (THREADS * 80) : 0;
 };
 
+// Two pencils, ky and ky + Ly / 2, share 2 TPC threads: each transforms its own,
+// then half-warps take turns over the two resampled spectra, so that a warp's
+// store fills two whole 128-byte lines of V, blocked or not (the half-warp of
+// a pencil covers 16 consecutive m). One pencil per warp, 32 consecutive m,
+// touched four half lines of the blocked layout per store, and the kernel,
+// whose L1 data path is its busiest unit (78 %), ran 353 us at 256x256x512
+// float32; this way 325 us (and 318 us with V unblocked, whose lateral inverse
+// then took 393 us against 350 us).
+// (16-bit storage, and transforms by fewer than 16 threads, keep one pencil
+// per thread group.)
 template <int L, int PPC, class TS, bool kRamp, int E>
 __global__ void __launch_bounds__(FkLiteTile<L, PPC, E>::THREADS, FkLiteTile<L, PPC, E>::MINB) fk_stolt_kernel(const FkZParams p) {
   using S = FftShape<L, E>;
   extern __shared__ float2 fl_sm[];
   const int w = threadIdx.x / S::TPC;
   const int j0 = threadIdx.x % S::TPC;
-  const long long pid = (long long)blockIdx.x * PPC + w;
-  const bool valid = pid < p.npencils;
-  const int twob = p.b_pad;
-  const int kx = valid ? (int)(pid / twob) : 0;
-  const int ky = valid ? (int)(pid % twob) : 0;
+  constexpr bool kPlaces = sizeof(TS) == 8;   // psi_pos order of the blocked layout
+  constexpr bool kPair = kPlaces && S::TPC >= 16 && PPC % 2 == 0;
+  const int twob = p.b_pad, hb = twob >> 1;
+  // this CTA's pencil v: pairs (u, u + hb) of one kx, or one after the other
+  auto pencil = [&](int v, int& kx, int& ky) {
+    const long long pid = (long long)blockIdx.x * PPC + v;
+    const bool ok = pid < p.npencils;
+    const long long q = !ok ? 0 : kPair ? pid >> 1 : pid;
+    kx = (int)(q / (kPair ? hb : twob));
+    ky = (int)(q % (kPair ? hb : twob)) + (kPair && ok ? (v & 1) * hb : 0);
+    return ok;
+  };
+  int kx, ky;
+  bool valid = pencil(w, kx, ky);
   float2* U = fl_sm + w * S::SMEM;
   const float ldmul = p.ld_scale * (p.ld_dev_scale ? *p.ld_dev_scale : 1.0f);
   {
-    const long long q = valid ? pid : 0;
+    const long long q = (long long)kx * twob + ky;
     FkLiteFwdCtx<L, TS, kRamp, E> ctx{static_cast<const TS*>(p.G) + q * p.n, U, E == 32 ? p.tw32 : p.tw, valid,
                                       ldmul, p.t_ramp, q * p.n, p.G_n, p.err};
     fftn_run<L, 1, true, false, FkLiteFwdCtx<L, TS, kRamp, E>, E>(ctx, j0);
   }
-  if constexpr (fk_lite_bar<L, E>() == 32) __syncwarp();
-  else __syncthreads();
+  int m0 = j0;   // first m of this thread
+  if constexpr (kPair) {
+    constexpr int PT = 2 * S::TPC;                    // threads of a pair: whole warps
+    if constexpr (fk_lite_bar<L, E>() == 32) {
+      // one named barrier per pair of warps (ids known to the compiler: an SM's barriers are few)
+      static_assert(PPC <= 8, "up to four pairs");
+      const int pr = w >> 1;
+      if (pr == 0) asm volatile("bar.sync 1, 64;" ::: "memory");
+      else if (PPC > 2 && pr == 1) asm volatile("bar.sync 2, 64;" ::: "memory");
+      else if (PPC > 4 && pr == 2) asm volatile("bar.sync 3, 64;" ::: "memory");
+      else if (PPC > 6) asm volatile("bar.sync 4, 64;" ::: "memory");
+    } else {
+      __syncthreads();
+    }
+    const int t = threadIdx.x % PT;
+    const int v = (w & ~1) + ((t >> 4) & 1);
+    valid = pencil(v, kx, ky);
+    U = fl_sm + v * S::SMEM;
+    m0 = (t >> 5) * 16 + (t & 15);
+  } else if constexpr (fk_lite_bar<L, E>() == 32) {
+    __syncwarp();
+  } else {
+    __syncthreads();
+  }
   if (!valid) return;
   const float2 ax = p.ax[kx];
   const float2 ay = p.ay[ky];
   float2 A = two_sum(ax.x, ay.x);
   A = fast_two_sum(A.x, A.y + (ax.y + ay.y));
   TS* V = static_cast<TS*>(p.psi);
-  const long long o0 = ((long long)kx * twob + ky) * p.n;
+  const long long o0 = (long long)kx * twob * p.n + (p.psi_blocked ? (long long)(kPlaces ? psi_pos(ky, hb) : ky) * 8 : (long long)ky * p.n);
   const int mkx = (kx == 0) ? 0 : p.a_pad - kx;
   const int mky = (twob - ky) & (twob - 1);
-  const long long o1 = ((long long)mkx * twob + mky) * p.n;
+  const long long o1 = (long long)mkx * twob * p.n + (p.psi_blocked ? (long long)(kPlaces ? psi_pos(mky, hb) : mky) * 8 : (long long)mky * p.n);
   // the partner is stored only where it is not itself a stored pencil
   const bool partner = kx > 0 && 2 * kx < p.a_pad;
   const float st = kRamp ? p.st_scale : p.st_scale * ldmul;
   const StoltSplitA As = stolt_split_a(A.x, A.y);
-  float fm = (float)j0;
-  for (int m = j0; m < L / 2; m += S::TPC, fm += (float)S::TPC) {
+  float fm = (float)m0;
+  // V's element m lies at (m / 8) s8 + m % 8: a constant step where the
+  // stride over m is whole blocks
+  constexpr bool kStep = S::TPC % 8 == 0;
+  const long long s8 = p.psi_blocked ? 8LL * twob : 8LL;
+  long long om = kStep ? (m0 >> 3) * s8 + (m0 & 7) : 0;
+  const long long step = (S::TPC / 8) * s8;
+#pragma unroll 4
+  for (int m = m0; m < L / 2; m += S::TPC, fm += (float)S::TPC) {
     float2 d = make_float2(0.f, 0.f), e = d;
     if (m >= 1) {
       const StoltCoord c = stolt_coord_split(As, m, fm, L / 2);
@@ -131,8 +179,10 @@ __global__ void __launch_bounds__(FkLiteTile<L, PPC, E>::THREADS, FkLiteTile<L, 
         e = make_float2(fmaf(b1, w1.x, b0 * w0.x), -fmaf(b1, w1.y, b0 * w0.y));
       }
     }
-    if (bchk(o0 + m, p.psi_n, p.err)) Cpx<TS>::put(V + o0 + m, d);
-    if (partner && bchk(o1 + m, p.psi_n, p.err)) Cpx<TS>::put(V + o1 + m, e);
+    if (!kStep) om = (m >> 3) * s8 + (m & 7);
+    if (bchk(o0 + om, p.psi_n, p.err)) Cpx<TS>::put(V + o0 + om, d);
+    if (partner && bchk(o1 + om, p.psi_n, p.err)) Cpx<TS>::put(V + o1 + om, e);
+    if (kStep) om += step;
   }
 }
 
@@ -182,6 +232,7 @@ __global__ void __launch_bounds__(FkLiteTile<L, PPC, E>::THREADS, FkLiteTile<L, 
 
 template <int L, int PPC, class TS, bool kRamp, int E = 16>
 cudaError_t launch_fk_stolt_one(const FkZParams& p, cudaStream_t s) {
+  if (p.npencils % 2 || p.b_pad % 2) return cudaErrorInvalidValue;   // pairs (u, u + b_pad / 2)
   using T = FkLiteTile<L, PPC, E>;
   auto k = fk_stolt_kernel<L, PPC, TS, kRamp, E>;
   if (T::SMEM > 48 * 1024) {

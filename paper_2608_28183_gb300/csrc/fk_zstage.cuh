@@ -76,6 +76,7 @@ struct FkInvCtx {
   int n_out;                 // kept outputs z < n_out
   long long off0, off1, psi_n;   // offsets of out0 / out1 in their buffer, its extent (bounds-checked build)
   int* err;
+  int s8;                    // stride of blocks of 8 outputs (kGuard)
   __device__ __forceinline__ void load(int m, float2 (&x)[2]) const {
     x[0] = x[1] = make_float2(0.f, 0.f);
     if (m < 1) return;                                // m < L/2 (upper half is pruned)
@@ -91,6 +92,9 @@ struct FkInvCtx {
   __device__ __forceinline__ float2* sm(int t) const { return t == 0 ? W0 : W1; }
   __device__ __forceinline__ void store(int l, const float2 (&x)[2]) const {   // every l the schedule keeps
     if (kGuard && l >= n_out) return;
+    // (plans with L = 2n and fused lateral stages take their inverse last:
+    // here psi is blocked by 8 columns only where the guard is on)
+    if (kGuard) l = (l >> 3) * s8 + (l & 7);
     if (st0 && bchk(off0 + l, psi_n, err)) Cpx<TS>::put(out0 + l, cscale(x[0], stmul));
     if (st1 && bchk(off1 + l, psi_n, err)) Cpx<TS>::put(out1 + l, cscale(x[1], stmul));
   }
@@ -152,13 +156,14 @@ fk_zstage_kernel(const FkZParams p) {
   float2 A = two_sum(ax.x, ay.x);
   A = fast_two_sum(A.x, A.y + (ax.y + ay.y));
   TS* psi = static_cast<TS*>(p.psi);
-  const long long o_direct = ((long long)kx * twob + ky) * p.n;
+  const bool blk = kGuard && p.psi_blocked;
+  const long long o_direct = (long long)kx * twob * p.n + (blk ? (long long)(sizeof(TS) == 8 ? psi_pos(ky, twob / 2) : ky) * 8 : (long long)ky * p.n);
   const int mkx = (kx == 0) ? 0 : p.a_pad - kx;
   const int mky = (twob - ky) & (twob - 1);
-  const long long o_mirror = ((long long)mkx * twob + mky) * p.n;
+  const long long o_mirror = (long long)mkx * twob * p.n + (blk ? (long long)(sizeof(TS) == 8 ? psi_pos(mky, twob / 2) : mky) * 8 : (long long)mky * p.n);
   // the partner is stored only where it is not itself a stored pencil
   FkInvCtx<L, TS, kAlias, kGuard> ctx{U, W0, W1, p.tw, psi + o_direct, psi + o_mirror, L / 2, A.x, A.y,
-                      valid, valid && kx > 0 && 2 * kx < p.a_pad, p.st_scale, p.n, o_direct, o_mirror, p.psi_n, p.err};
+                      valid, valid && kx > 0 && 2 * kx < p.a_pad, p.st_scale, p.n, o_direct, o_mirror, p.psi_n, p.err, blk ? 8 * twob : 8};
   fftn_run<L, 2, true, kPad2>(ctx, j0);
 }
 

@@ -79,6 +79,7 @@ struct FkWarpInvCtx {
   int n_out;
   long long out_off, psi_n;  // offset of out in its buffer, the buffer's extent (bounds-checked build)
   int* err;
+  int s8;                    // stride of blocks of 8 outputs (kGuard)
   __device__ __forceinline__ void load(int m, float2 (&x)[1]) const {
     x[0] = make_float2(0.f, 0.f);
     const unsigned e = coord[m];                  // m < L/2: the upper half is pruned
@@ -102,6 +103,7 @@ struct FkWarpInvCtx {
   __device__ __forceinline__ float2* sm(int) const { return buf; }
   __device__ __forceinline__ void store(int l, const float2 (&x)[1]) const {
     if (kGuard && l >= n_out) return;
+    if (kGuard) l = (l >> 3) * s8 + (l & 7);
     if (st && bchk(out_off + l, psi_n, err)) Cpx<TS>::put(out + l, cscale(x[0], stmul));
   }
 };
@@ -153,9 +155,11 @@ __global__ void __launch_bounds__(64) fk_zwarp_kernel(const FkZParams p) {
   __syncthreads();   // the table, and each warp's spectrum
   TS* psi = static_cast<TS*>(p.psi);
   const bool own = w == 0 || !single;
+  const bool blk = kGuard && p.psi_blocked;
   {
-    FkWarpInvCtx<L, TS, kGuard, false> ctx{U, W, coord, jac, p.tw32, psi + pid * p.n, own, p.st_scale, p.n, pid * p.n,
-                                           p.psi_n, p.err};
+    const long long o = (long long)kx * p.b_pad * p.n + (blk ? (long long)(sizeof(TS) == 8 ? psi_pos(ky, p.b_pad / 2) : ky) * 8 : (long long)ky * p.n);
+    FkWarpInvCtx<L, TS, kGuard, false> ctx{U, W, coord, jac, p.tw32, psi + o, own, p.st_scale, p.n, o,
+                                           p.psi_n, p.err, blk ? 8 * p.b_pad : 8};
     fftn_run<L, 1, true, kPad2, FkWarpInvCtx<L, TS, kGuard, false>, 32>(ctx, lane);
   }
   {
@@ -163,8 +167,8 @@ __global__ void __launch_bounds__(64) fk_zwarp_kernel(const FkZParams p) {
     const int mkx = (kx == 0) ? 0 : p.a_pad - kx;
     const int mky = (p.b_pad - ky) & (p.b_pad - 1);
     const bool st = own && kx > 0 && 2 * kx < p.a_pad;
-    const long long mo = ((long long)mkx * p.b_pad + mky) * p.n;
-    FkWarpInvCtx<L, TS, kGuard, true> ctx{U, U, coord, jac, p.tw32, psi + mo, st, p.st_scale, p.n, mo, p.psi_n, p.err};
+    const long long mo = (long long)mkx * p.b_pad * p.n + (blk ? (long long)(sizeof(TS) == 8 ? psi_pos(mky, p.b_pad / 2) : mky) * 8 : (long long)mky * p.n);
+    FkWarpInvCtx<L, TS, kGuard, true> ctx{U, U, coord, jac, p.tw32, psi + mo, st, p.st_scale, p.n, mo, p.psi_n, p.err, blk ? 8 * p.b_pad : 8};
     fftn_run<L, 1, true, kPad2, FkWarpInvCtx<L, TS, kGuard, true>, 32>(ctx, lane);
   }
 }

@@ -781,7 +781,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
     ch.nchunks = (int)(n / 16);
     ch.sync = sync;
     ch.err = err;
-    ch.discard = 0;   // per stage below (variant 0 on float32 storage)
+    ch.discard = 0;   // per stage below
   }
   AxisLaunch l{};
   if (part == 2) {
@@ -800,15 +800,14 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
     c.p.in_n = a * b * n;
     c.p.mid_n = ws_extent(p, 0);
     c.p.out_n = ws_extent(p, 1);
-    c.p.discard = st == kF32 && p->tiles[sid] < 2;
+    c.p.discard = p->tiles[sid] < 2;
     c.nslot = p->tiles[sid] % 2 == 0 ? 3 : 2;
     c.fwd = 1;
-    // x items: 16 real t columns of one wall row, a rows; y items: 8 complex columns of one kx, b rows
+    // x items: 16 real t columns of one wall row, a rows
     // no L2 promotion: a wider fetch would pull in the next chunks' columns, whose
     // items come hundreds of tickets later (evicted by then, read twice)
-    if (!encode_3d(&c.map1, H, rb, (unsigned long long)(b * n), a, 1, b * n * rb, a * b * n * rb, 16,
-                   (unsigned)std::min<long long>(a, 256), false) ||
-        !encode_3d(&c.map2, b0, cb, n, b, hx, n * cb, b * n * cb, 8, (unsigned)std::min<long long>(b, 256), false))
+    if (!encode_3d(&c.map, H, rb, (unsigned long long)(b * n), a, 1, b * n * rb, a * b * n * rb, 16,
+                   (unsigned)std::min<long long>(a, 256), false))
       return fail(NLOS_ERR_CUDA, "fk xy-forward: tensor map encoding failed");
     NLOS_CU(cudaMemsetAsync(sync, 0, sync_bytes, s), "fk chain counters");
     NLOS_CU(launch_fk_chain(c, st, s), "fk xy-forward");
@@ -857,6 +856,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
   z.t_ramp = part == 2 ? ramp : 0.0f;
   z.G_n = ws_extent(p, 1);
   z.psi_n = ws_extent(p, 2);
+  z.psi_blocked = p->fused ? 1 : 0;
   z.err = err;
   if (p->zlast) {
     // FK3 without its inverses: the resampled spectra of both partners
@@ -874,14 +874,10 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
     c.p.in_n = ws_extent(p, 2);
     c.p.mid_n = ws_extent(p, 0);
     c.p.out_n = std::min<long long>(ws_extent(p, 1), a * b * n);
-    c.p.discard = st == kF32 && p->tiles[sid] < 2;
+    c.p.discard = p->tiles[sid] < 2;
     c.nslot = p->tiles[sid] % 2 == 0 ? 3 : 2;
     c.fwd = 0;
     c.store_mode = kStoreCpx;   // the storage type
-    const unsigned box = (unsigned)std::min<long long>(Lx, 256);
-    if (!encode_3d(&c.map1, b2, cb, n, Ly, Lx, n * cb, Ly * n * cb, 8, box, false) ||
-        !encode_3d(&c.map2, b0, cb, n, Lx, b, b * n * cb, n * cb, 8, box, false))
-      return fail(NLOS_ERR_CUDA, "fk yx-inverse: tensor map encoding failed");
     NLOS_CU(cudaMemsetAsync(sync, 0, sync_bytes, s), "fk chain counters");
     NLOS_CU(launch_fk_chain(c, st, s), "fk yx-inverse");
     NLOS_MARK(p, s, sid++);
@@ -921,15 +917,10 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
     c.p.in_n = ws_extent(p, 2);
     c.p.mid_n = ws_extent(p, 0);
     c.p.out_n = a * b * n;
-    c.p.discard = st == kF32 && p->tiles[sid] < 2;
+    c.p.discard = p->tiles[sid] < 2;
     c.nslot = p->tiles[sid] % 2 == 0 ? 3 : 2;
     c.fwd = 0;
     c.store_mode = cpx ? kStoreCpx32 : kStoreAbs2;
-    // y items: 8 complex columns of one kx, Ly rows; x items: 8 complex columns of one wall row y, Lx rows
-    const unsigned box = (unsigned)std::min<long long>(Lx, 256);
-    if (!encode_3d(&c.map1, b2, cb, n, Ly, Lx, n * cb, Ly * n * cb, 8, box, false) ||
-        !encode_3d(&c.map2, b0, cb, n, Lx, b, b * n * cb, n * cb, 8, box, false))
-      return fail(NLOS_ERR_CUDA, "fk yx-inverse: tensor map encoding failed");
     NLOS_CU(cudaMemsetAsync(sync, 0, sync_bytes, s), "fk chain counters");
     NLOS_CU(launch_fk_chain(c, st, s), "fk yx-inverse");
     NLOS_MARK(p, s, sid++);

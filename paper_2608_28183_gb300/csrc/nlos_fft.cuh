@@ -226,6 +226,16 @@ template <class C> struct CtxInverse<C, decltype((void)C::kInverse)> {
   static constexpr bool value = C::kInverse;
 };
 
+// Contexts whose input is permuted by the position of l = j + r Q in the first
+// pass (row r of R, j < Q) declare kLoadRow and provide
+// load_row(int j, int r, int Q, int R, float2 (&x)[NT]) instead of load(l).
+template <class C, class = void> struct CtxLoadRow {
+  static constexpr bool value = false;
+};
+template <class C> struct CtxLoadRow<C, decltype((void)C::kLoadRow)> {
+  static constexpr bool value = C::kLoadRow;
+};
+
 template <class Ctx> __device__ __forceinline__ void fft_sync() {
   if constexpr (CtxBar<Ctx>::threads == 0) {
     __syncthreads();
@@ -275,7 +285,8 @@ __device__ __forceinline__ void fftn_passes(Ctx& ctx, const int j0, float2 (&v)[
           for (int t = 0; t < NT; ++t) v[t][i * R + r] = make_float2(0.f, 0.f);
         } else {
           float2 x[NT];
-          ctx.load(j + r * Q, x);
+          if constexpr (CtxLoadRow<Ctx>::value) ctx.load_row(j, r, Q, R, x);
+          else ctx.load(j + r * Q, x);
 #pragma unroll
           for (int t = 0; t < NT; ++t) v[t][i * R + r] = x[t];
         }

@@ -78,11 +78,26 @@ constexpr int kDevErrBounds = 3;          // bounds-checked build: an index outs
 __host__ __device__ constexpr int fk_tile_count(int L) { return L == 1024 ? 5 : 4; }
 __host__ __device__ constexpr int fk_tile_default(int L) { return L == 1024 ? 2 : 0; }
 
+// Place of ky in a block of the fused lateral inverse's float32 input: ky and
+// ky + h (h = Ly / 2) share a pair of places, one 128-byte line, and odd pairs
+// hold them swapped. Negation maps such pairs onto each other, so the two
+// pencils of a pair, and their Hermitian partners, fill whole lines; and the
+// first pass of the inverse, which reads ky and ky + 1 side by side, finds
+// them in different halves of the banks. (16-bit values gain nothing from
+// it: their rows are 32 bytes, and the Stolt stage ran 297 us against 293 at
+// 256x256x512.)
+__host__ __device__ constexpr int psi_pos(int ky, int h) {
+  return ((ky & (h - 1)) << 1) | ((ky >= h ? 1 : 0) ^ (ky & 1));
+}
+
 // f-k temporal-frequency stage: forward length-2n FFT of each stored pencil
 // G[kx][ky][0..n) (kx in [0, a], ky in [0, 2b)), Stolt resampling with the
 // Jacobian and the Z > 0 mask, and inverse length-2n FFTs producing the pencil
 // (kx, ky) and, for 0 < kx < a, its Hermitian partner (2a-kx, -ky), keeping
-// z < n. Output psi[kx'][ky'][z] for kx' in [0, 2a).
+// z < n. Output psi of kx' in [0, 2a): value z of pencil (kx', ky') lies at
+// kx' * b_pad * n + ky' * n + z, or (psi_blocked) blocked by 8 columns for the
+// fused lateral inverse: [kx'][z / 8][place of ky'][z % 8], where the place is
+// psi_pos(ky', b_pad / 2) for float32 storage and ky' for 16-bit storage.
 struct FkZParams {
   const void* G;
   void* psi;
@@ -97,6 +112,7 @@ struct FkZParams {
   float ld_scale;              // multiplies forward loads
   const float* ld_dev_scale;   // optional device scalar multiplying forward loads
   float st_scale;              // multiplies stored values
+  int psi_blocked;             // layout of psi (see above)
   float t_ramp;                // non-zero: forward loads also multiplied by t * t_ramp (the
                                // spectrum was taken without the t/(n-1) ramp; float32 only,
                                // launch shape 0 whatever `tile` asks)
@@ -125,10 +141,13 @@ struct FkZInvParams {
 cudaError_t launch_fk_zinv(const FkZInvParams& p, int storage, int tile, cudaStream_t s);
 
 // f-k lateral transforms fused in pairs (fk_chain.cuh):
-//   forward: in = H [a][b][n] real, mid = [L/2 + 1][b][n], out = G [L/2 + 1][L][n]
-//   inverse: in = psi [L][L][n], mid = [L][b][n], out = [a][b][n] float
-//            (|.|^2), float2 (complex) or the storage type (complex, the
-//            spectrum whose temporal inverse comes last)
+//   forward: in = H [a][b][n] real, mid = [n/8][L/2 + 1][b][8], out = G [L/2 + 1][L][n]
+//   inverse: in = psi [L][n/8][L][8] (kx, block of 8 columns, place of ky, column),
+//            mid = [n/8][b][L][8], out = [a][b][n] float (|.|^2), float2
+//            (complex) or the storage type (complex, the spectrum whose
+//            temporal inverse comes last)
+// psi and mid are blocked by 8 columns so that a sub-tile of 8 columns over a
+// whole transformed axis is one contiguous run of memory.
 struct FkChainParams {
   const void* in;
   void* mid;
@@ -148,7 +167,7 @@ struct FkChainParams {
 };
 struct FkChainLaunch {
   FkChainParams p;
-  CUtensorMap map1, map2;      // TMA maps of the first / second transform's input
+  CUtensorMap map;             // forward: TMA map of the transient
   int fwd;                     // 1 forward, 0 inverse
   int store_mode;              // inverse: kStoreAbs2 or kStoreCpx32
   int nslot;                   // shared-memory slots per CTA (2 or 3; 2 at L = 1024)

@@ -92,6 +92,17 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
+// Contiguous bulk copy of `bytes` (a multiple of 16, both addresses 16-byte
+// aligned) into shared memory with an L2 cache-eviction policy, completing on `bar`.
+__device__ __forceinline__ void bulk_load_hint(void* dst, const void* src, uint32_t bytes, uint64_t* bar,
+                                               uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
+          smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
+      : "memory");
+}
+
 // L2 policy for data read exactly once: its lines are the first to go
 __device__ __forceinline__ uint64_t l2_policy_evict_first() {
   uint64_t pol;
