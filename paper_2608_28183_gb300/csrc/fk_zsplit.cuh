@@ -23,7 +23,9 @@
 // 3 (a + 1) 2b to (a + 1) 2b + a b per volume, for 24V more bytes moved
 // (V's 32V written and read once more at a quarter of its size: 8V, plus the
 // complex intermediate of FK4). Any storage type (the 16-bit forms keep the
-// per-pass scales of the other stages), L = 2n.
+// per-pass scales of the other stages) for L = 2n; float32 storage for longer
+// L as well (a time axis that is not a power of two), where V has L / 2
+// columns and the lateral inverses run over those instead of n.
 #pragma once
 #include "fk_stolt.cuh"
 #include "fk_zstage.cuh"
@@ -43,7 +45,8 @@ template <int L, int E> constexpr int fk_lite_bar() { return FftShape<L, E>::TPC
 // pass stores the spectrum unpadded, U[l]: its lanes write consecutive l, and
 // the Stolt gather then indexes U without the padding arithmetic. The load
 // scale of the non-ramped form is applied after the transform (it is linear).
-template <int L, class TS, bool kRamp, int E>
+// kGuard: the pencil has fewer than L / 2 samples (n_in), the rest reads zero
+template <int L, class TS, bool kRamp, bool kGuard, int E>
 struct FkLiteFwdCtx {
   static constexpr int SSTRIDE = 1;
   static constexpr bool kSmemInput = false;
@@ -53,10 +56,11 @@ struct FkLiteFwdCtx {
   const float2* tw;
   bool valid;
   float ldmul, t_ramp;
+  int n_in;
   long long g_off, g_n;
   int* err;
   __device__ __forceinline__ void load(int l, float2 (&x)[1]) const {
-    if (!(valid && bchk(g_off + l, g_n, err))) {
+    if (!(valid && (!kGuard || l < n_in) && bchk(g_off + l, g_n, err))) {
       x[0] = make_float2(0.f, 0.f);
     } else if constexpr (kRamp) {
       x[0] = cscale(Cpx<TS>::get(g + l), ldmul * (float)l * t_ramp);
@@ -89,7 +93,7 @@ template <int L, int PPC, int E> struct FkLiteTile {
 // then took 393 us against 350 us).
 // (16-bit storage, and transforms by fewer than 16 threads, keep one pencil
 // per thread group.)
-template <int L, int PPC, class TS, bool kRamp, int E>
+template <int L, int PPC, class TS, bool kRamp, bool kGuard, int E>
 __global__ void __launch_bounds__(FkLiteTile<L, PPC, E>::THREADS, FkLiteTile<L, PPC, E>::MINB) fk_stolt_kernel(const FkZParams p) {
   using S = FftShape<L, E>;
   extern __shared__ float2 fl_sm[];
@@ -113,9 +117,10 @@ __global__ void __launch_bounds__(FkLiteTile<L, PPC, E>::THREADS, FkLiteTile<L, 
   const float ldmul = p.ld_scale * (p.ld_dev_scale ? *p.ld_dev_scale : 1.0f);
   {
     const long long q = (long long)kx * twob + ky;
-    FkLiteFwdCtx<L, TS, kRamp, E> ctx{static_cast<const TS*>(p.G) + q * p.n, U, E == 32 ? p.tw32 : p.tw, valid,
-                                      ldmul, p.t_ramp, q * p.n, p.G_n, p.err};
-    fftn_run<L, 1, true, false, FkLiteFwdCtx<L, TS, kRamp, E>, E>(ctx, j0);
+    using Ctx = FkLiteFwdCtx<L, TS, kRamp, kGuard, E>;
+    Ctx ctx{static_cast<const TS*>(p.G) + q * p.n, U, E == 32 ? p.tw32 : p.tw, valid,
+            ldmul, p.t_ramp, p.n, q * p.n, p.G_n, p.err};
+    fftn_run<L, 1, true, false, Ctx, E>(ctx, j0);
   }
   int m0 = j0;   // first m of this thread
   if constexpr (kPair) {
@@ -147,10 +152,12 @@ __global__ void __launch_bounds__(FkLiteTile<L, PPC, E>::THREADS, FkLiteTile<L, 
   float2 A = two_sum(ax.x, ay.x);
   A = fast_two_sum(A.x, A.y + (ax.y + ay.y));
   TS* V = static_cast<TS*>(p.psi);
-  const long long o0 = (long long)kx * twob * p.n + (p.psi_blocked ? (long long)(kPlaces ? psi_pos(ky, hb) : ky) * 8 : (long long)ky * p.n);
+  const long long o0 = (long long)kx * twob * (L / 2) +
+                       (p.psi_blocked ? (long long)(kPlaces ? psi_pos(ky, hb) : ky) * 8 : (long long)ky * (L / 2));
   const int mkx = (kx == 0) ? 0 : p.a_pad - kx;
   const int mky = (twob - ky) & (twob - 1);
-  const long long o1 = (long long)mkx * twob * p.n + (p.psi_blocked ? (long long)(kPlaces ? psi_pos(mky, hb) : mky) * 8 : (long long)mky * p.n);
+  const long long o1 = (long long)mkx * twob * (L / 2) +
+                       (p.psi_blocked ? (long long)(kPlaces ? psi_pos(mky, hb) : mky) * 8 : (long long)mky * (L / 2));
   // the partner is stored only where it is not itself a stored pencil
   const bool partner = kx > 0 && 2 * kx < p.a_pad;
   const float st = kRamp ? p.st_scale : p.st_scale * ldmul;
@@ -187,8 +194,8 @@ __global__ void __launch_bounds__(FkLiteTile<L, PPC, E>::THREADS, FkLiteTile<L, 
 }
 
 // inverse temporal transform of a kept pencil: input m < L/2 (the upper half
-// is zero), output z < L/2
-template <int L, class TS, bool kCpx, int E>
+// is zero), output z < L/2 (kGuard: z < n_out)
+template <int L, class TS, bool kCpx, bool kGuard, int E>
 struct FkZInvCtx {
   static constexpr int SSTRIDE = 1;
   static constexpr bool kInverse = true;
@@ -200,6 +207,7 @@ struct FkZInvCtx {
   const float2* tw;
   bool valid;
   float scale;
+  int n_out;
   long long in_off, in_n, out_off, out_n;
   int* err;
   __device__ __forceinline__ void load(int l, float2 (&x)[1]) const {
@@ -207,13 +215,13 @@ struct FkZInvCtx {
   }
   __device__ __forceinline__ float2* sm(int) const { return W; }
   __device__ __forceinline__ void store(int l, const float2 (&x)[1]) const {
-    if (!valid || !bchk(out_off + l, out_n, err)) return;
+    if (!valid || (kGuard && l >= n_out) || !bchk(out_off + l, out_n, err)) return;
     if (kCpx) static_cast<float2*>(out)[l] = cscale(x[0], scale);
     else static_cast<float*>(out)[l] = scale * fmaf(x[0].x, x[0].x, x[0].y * x[0].y);
   }
 };
 
-template <int L, int PPC, class TS, bool kCpx, int E>
+template <int L, int PPC, class TS, bool kCpx, bool kGuard, int E>
 __global__ void __launch_bounds__(FkLiteTile<L, PPC, E>::THREADS, FkLiteTile<L, PPC, E>::MINB) fk_zinv_kernel(const FkZInvParams p) {
   using S = FftShape<L, E>;
   extern __shared__ float2 zi_sm[];
@@ -225,16 +233,38 @@ __global__ void __launch_bounds__(FkLiteTile<L, PPC, E>::THREADS, FkLiteTile<L, 
   void* out = kCpx ? static_cast<void*>(static_cast<float2*>(p.out) + q * p.n)
                    : static_cast<void*>(static_cast<float*>(p.out) + q * p.n);
   const float scale = p.scale * (p.dev_scale ? *p.dev_scale : 1.0f);
-  FkZInvCtx<L, TS, kCpx, E> ctx{static_cast<const TS*>(p.in) + q * p.n, out, zi_sm + w * S::SMEM,
-                             E == 32 ? p.tw32 : p.tw, valid, scale, q * p.n, p.in_n, q * p.n, p.out_n, p.err};
-  fftn_run<L, 1, true, true, FkZInvCtx<L, TS, kCpx, E>, E>(ctx, j0);
+  using Ctx = FkZInvCtx<L, TS, kCpx, kGuard, E>;
+  Ctx ctx{static_cast<const TS*>(p.in) + q * (L / 2), out, zi_sm + w * S::SMEM, E == 32 ? p.tw32 : p.tw, valid, scale, p.n,
+          q * (L / 2), p.in_n, q * p.n, p.out_n, p.err};
+  fftn_run<L, 1, true, true, Ctx, E>(ctx, j0);
 }
 
-template <int L, int PPC, class TS, bool kRamp, int E = 16>
-cudaError_t launch_fk_stolt_one(const FkZParams& p, cudaStream_t s) {
+template <int L, int PPC, class TS, bool kRamp, bool kGuard, int E>
+cudaError_t launch_fk_stolt_as(const FkZParams& p, cudaStream_t s) {
   if (p.npencils % 2 || p.b_pad % 2) return cudaErrorInvalidValue;   // pairs (u, u + b_pad / 2)
   using T = FkLiteTile<L, PPC, E>;
-  auto k = fk_stolt_kernel<L, PPC, TS, kRamp, E>;
+  auto k = fk_stolt_kernel<L, PPC, TS, kRamp, kGuard, E>;
+  if (T::SMEM > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::SMEM);
+    if (e != cudaSuccess) return e;
+  }
+  const long long blocks = (p.npencils + PPC - 1) / PPC;
+  k<<<(unsigned)blocks, T::THREADS, T::SMEM, s>>>(p);
+  return cudaGetLastError();
+}
+
+// L > 2n: float32 storage only
+template <int L, int PPC, class TS, bool kRamp, int E = 16>
+cudaError_t launch_fk_stolt_one(const FkZParams& p, cudaStream_t s) {
+  if (p.n == L / 2) return launch_fk_stolt_as<L, PPC, TS, kRamp, false, E>(p, s);
+  if constexpr (sizeof(TS) == 8) return launch_fk_stolt_as<L, PPC, TS, kRamp, true, E>(p, s);
+  else return cudaErrorInvalidValue;
+}
+
+template <int L, int PPC, class TS, bool kCpx, bool kGuard, int E>
+cudaError_t launch_fk_zinv_as(const FkZInvParams& p, cudaStream_t s) {
+  using T = FkLiteTile<L, PPC, E>;
+  auto k = fk_zinv_kernel<L, PPC, TS, kCpx, kGuard, E>;
   if (T::SMEM > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::SMEM);
     if (e != cudaSuccess) return e;
@@ -246,23 +276,18 @@ cudaError_t launch_fk_stolt_one(const FkZParams& p, cudaStream_t s) {
 
 template <int L, int PPC, class TS, bool kCpx, int E = 16>
 cudaError_t launch_fk_zinv_one(const FkZInvParams& p, cudaStream_t s) {
-  using T = FkLiteTile<L, PPC, E>;
-  auto k = fk_zinv_kernel<L, PPC, TS, kCpx, E>;
-  if (T::SMEM > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::SMEM);
-    if (e != cudaSuccess) return e;
-  }
-  const long long blocks = (p.npencils + PPC - 1) / PPC;
-  k<<<(unsigned)blocks, T::THREADS, T::SMEM, s>>>(p);
-  return cudaGetLastError();
+  if (p.n == L / 2) return launch_fk_zinv_as<L, PPC, TS, kCpx, false, E>(p, s);
+  if constexpr (sizeof(TS) == 8) return launch_fk_zinv_as<L, PPC, TS, kCpx, true, E>(p, s);
+  else return cudaErrorInvalidValue;
 }
 
 // launch shapes 0 / 1: radix-16 passes at the two pencils-per-CTA counts of
 // fk_ppc; 2 / 3: radix-32 passes (32 values per thread) at twice those
-// counts (the same threads per CTA). The ramped form, float32 only, takes shape 0.
+// counts (the same threads per CTA; at L = 8192 shape 3 is one pencil per CTA,
+// three CTAs of 68 KB on an SM). The ramped form, float32 only, takes shape 0.
 template <int L, class TS>
 cudaError_t launch_fk_stolt_len(const FkZParams& p, int tile, cudaStream_t s) {
-  constexpr int P0 = fk_ppc(L, 0), P1 = fk_ppc(L, 1);
+  constexpr int P0 = fk_ppc(L, 0), P1 = fk_ppc(L, 1), P1X = L >= 8192 ? 1 : 2 * P1;
   if (p.t_ramp != 0.f) {
     if constexpr (std::is_same<TS, float2>::value) return launch_fk_stolt_one<L, P0, TS, true>(p, s);
     else return cudaErrorInvalidValue;
@@ -270,26 +295,26 @@ cudaError_t launch_fk_stolt_len(const FkZParams& p, int tile, cudaStream_t s) {
   switch (tile) {
     case 1: return launch_fk_stolt_one<L, P1, TS, false>(p, s);
     case 2: return launch_fk_stolt_one<L, 2 * P0, TS, false, 32>(p, s);
-    case 3: return launch_fk_stolt_one<L, 2 * P1, TS, false, 32>(p, s);
+    case 3: return launch_fk_stolt_one<L, P1X, TS, false, 32>(p, s);
     default: return launch_fk_stolt_one<L, P0, TS, false>(p, s);
   }
 }
 
 template <int L, class TS>
 cudaError_t launch_fk_zinv_len(const FkZInvParams& p, int tile, cudaStream_t s) {
-  constexpr int P0 = fk_ppc(L, 0), P1 = fk_ppc(L, 1);
+  constexpr int P0 = fk_ppc(L, 0), P1 = fk_ppc(L, 1), P1X = L >= 8192 ? 1 : 2 * P1;
   if (p.complex_out) {
     switch (tile) {
       case 1: return launch_fk_zinv_one<L, P1, TS, true>(p, s);
       case 2: return launch_fk_zinv_one<L, 2 * P0, TS, true, 32>(p, s);
-      case 3: return launch_fk_zinv_one<L, 2 * P1, TS, true, 32>(p, s);
+      case 3: return launch_fk_zinv_one<L, P1X, TS, true, 32>(p, s);
       default: return launch_fk_zinv_one<L, P0, TS, true>(p, s);
     }
   }
   switch (tile) {
     case 1: return launch_fk_zinv_one<L, P1, TS, false>(p, s);
     case 2: return launch_fk_zinv_one<L, 2 * P0, TS, false, 32>(p, s);
-    case 3: return launch_fk_zinv_one<L, 2 * P1, TS, false, 32>(p, s);
+    case 3: return launch_fk_zinv_one<L, P1X, TS, false, 32>(p, s);
     default: return launch_fk_zinv_one<L, P0, TS, false>(p, s);
   }
 }

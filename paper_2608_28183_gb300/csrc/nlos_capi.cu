@@ -75,7 +75,8 @@ cudaError_t launch_fk_stolt(const FkZParams& p, int storage, int tile, cudaStrea
       {launch_fk_stolt_f32_r0, launch_fk_stolt_f32_r1},
       {launch_fk_stolt_f16_r0, launch_fk_stolt_f16_r1},
       {launch_fk_stolt_bf16_r0, launch_fk_stolt_bf16_r1}};
-  if (p.npencils <= 0 || p.L != 2 * p.n || p.pad != 2 || storage < 0 || storage > 2) return cudaErrorInvalidValue;
+  if (p.npencils <= 0 || p.L < 2 * p.n || (p.L != 2 * p.n && storage != kF32) || p.pad != 2 || storage < 0 || storage > 2)
+    return cudaErrorInvalidValue;
   return fn[storage][p.L <= 1024 ? 0 : 1](p, tile, s);
 }
 
@@ -84,7 +85,8 @@ cudaError_t launch_fk_zinv(const FkZInvParams& p, int storage, int tile, cudaStr
       {launch_fk_zinv_f32_r0, launch_fk_zinv_f32_r1},
       {launch_fk_zinv_f16_r0, launch_fk_zinv_f16_r1},
       {launch_fk_zinv_bf16_r0, launch_fk_zinv_bf16_r1}};
-  if (p.npencils <= 0 || p.L != 2 * p.n || storage < 0 || storage > 2) return cudaErrorInvalidValue;
+  if (p.npencils <= 0 || p.L < 2 * p.n || (p.L != 2 * p.n && storage != kF32) || storage < 0 || storage > 2)
+    return cudaErrorInvalidValue;
   return fn[storage][p.L <= 1024 ? 0 : 1](p, tile, s);
 }
 
@@ -201,8 +203,11 @@ struct nlos_plan_s {
   size_t off[3] = {0, 0, 0};
   size_t off_scal = 0, off_part = 0;
   size_t off_sync = 0;                  // chunk counters of the fused lateral f-k stages
-  bool fused = false;                   // f-k lateral transforms fused in pairs (fk_chain.cuh)
+  bool fused = false;                   // f-k lateral forward transforms fused (fk_chain.cuh)
+  bool fused_inv = false;               // f-k lateral inverse transforms fused
   bool zlast = false;                   // f-k inverse temporal transform last (fk_zsplit.cuh)
+  int zcols = 0;                        // columns (m or z) the f-k lateral inverses run over
+  bool injected = false;                // an allocation failed through the testing hook
   size_t ws_bytes = 0;
   void* ws = nullptr;
   // host-call staging
@@ -238,6 +243,7 @@ nlos_status_t dalloc(nlos_plan_s* p, void** ptr, size_t bytes, const char* what)
   }
   if (k == 1) {
     *ptr = nullptr;
+    p->injected = true;
     return fail(NLOS_ERR_OUT_OF_MEMORY, "%s: injected allocation failure", what);
   }
   cudaError_t e = cudaMalloc(ptr, bytes ? bytes : 16);
@@ -310,6 +316,57 @@ float2 split_ff(double v) {
 // (Alg. 1's s per axis), signed index p~ of the Lx-point padded axis; for
 // Lx = 2a, Lt = 2n this is Alg. 1's (n s_x p~ / a)^2.
 // ---------------------------------------------------------------------------
+//
+// Workspace buffers of an f-k plan, in bytes. Temporal inverse inside the
+// stage, or last with L = 2n: b0 holds the x-transformed transient, then the
+// y-inverted spectrum; b1 G (kx <= Lx/2), then (last) the kept spectrum S;
+// b2 psi or V. Last with longer L: V (b2) has L/2 columns, so to stay small
+// the y-inverted spectrum takes G's place in b1 (dead by then) and S shares
+// b0 with the x-transformed transient.
+bool fk_wide(const nlos_plan_s* p) { return p->Lt > 2 * p->n; }
+void fk_buffers(const nlos_plan_s* p, bool zlast, size_t* b0, size_t* b1, size_t* b2) {
+  const size_t cb = complex_bytes(p->storage);
+  const size_t a = p->a, b = p->b, n = p->n, Lx = p->Lx, Ly = p->Ly, hx = Lx / 2 + 1;
+  if (zlast && fk_wide(p)) {
+    const size_t m = p->Lt / 2;
+    *b0 = std::max(hx * b * n, a * b * m) * cb;
+    *b1 = std::max(hx * Ly * n, Lx * b * m) * cb;
+    *b2 = Lx * Ly * m * cb;
+    return;
+  }
+  *b0 = Lx * b * n * cb;
+  *b1 = hx * Ly * n * cb;
+  *b2 = Lx * Ly * n * cb;
+}
+
+// Stage structure of an f-k plan. The fused lateral stages and L = 2n imply
+// the temporal inverse last, for every storage type. Float32 plans of other
+// shapes take it too, with the fused lateral inverse where the padded grid is
+// square, when
+//  * their buffers exceed 32 MiB: below that a volume takes a few launches of
+//    a few microseconds each and one stage more costs what it saves (and
+//    plans that fit nlos_reconstruct_noalloc's fixed scratch keep fitting);
+//  * their buffers grow by at most half (V has L/2 >= n columns).
+// Measured: 190x190x3002 13.99 -> 8.12 ms, 96x80x300 269 -> 216 us. 16-bit plans
+// keep their order of roundings.
+void fk_structure(nlos_plan_s* p, int flags) {
+  const auto& d = p->d;
+  const bool sep = flags & NLOS_PLAN_SEPARATE_AXES;
+  p->fused = !sep && fk_chain_eligible(p->a, p->b, p->n, p->Lx, p->Ly, d.pad_factor);
+  p->fused_inv = p->fused;
+  p->zlast = p->fused && !fk_wide(p);
+  p->zcols = p->n;
+  if (p->zlast || sep || d.pad_factor != 2 || p->storage != kF32 || (flags & kPlanSmallWorkspace)) return;
+  size_t o[3], w[3];
+  fk_buffers(p, false, &o[0], &o[1], &o[2]);
+  fk_buffers(p, true, &w[0], &w[1], &w[2]);
+  const size_t old_bytes = o[0] + o[1] + o[2], new_bytes = w[0] + w[1] + w[2];
+  if (old_bytes <= (size_t(32) << 20) || 2 * new_bytes > 3 * old_bytes) return;
+  p->zlast = true;
+  p->zcols = p->Lt / 2;
+  p->fused_inv = fk_chain_inv_eligible(p->zcols, p->Lx, p->Ly);
+}
+
 nlos_status_t build_fk(nlos_plan_s* p) {
   const auto& d = p->d;
   const int Lx = p->Lx, Ly = p->Ly, Lt = p->Lt;
@@ -334,18 +391,15 @@ nlos_status_t build_fk(nlos_plan_s* p) {
   if ((st = ensure_twiddles(p, Lx)) != NLOS_OK) return st;
   if ((st = ensure_twiddles(p, Ly)) != NLOS_OK) return st;
   if ((st = ensure_twiddles(p, Lt)) != NLOS_OK) return st;
-  const size_t cb = complex_bytes(p->storage);
-  const long long b = p->b, n = p->n, hx = Lx / 2 + 1;
-  const size_t b0 = std::max(hx * b * n, (long long)Lx * b * n) * cb;   // G1, then the y-inverse output
-  const size_t b1 = hx * Ly * n * cb;                                    // G (kx <= Lx/2)
-  const size_t b2 = (size_t)Lx * Ly * n * cb;                             // psi_z
+  size_t b0, b1, b2;
+  fk_buffers(p, p->zlast, &b0, &b1, &b2);
   p->off[0] = 0;
   p->off[1] = align256(b0);
   p->off[2] = p->off[1] + align256(b1);
   p->off_scal = p->off[2] + align256(b2);
   p->off_part = p->off_scal + 256;
   p->off_sync = p->off_part + align256(sizeof(float) * kScalePartials);
-  p->ws_bytes = p->off_sync + align256(sizeof(int) * (2 + n / 16));
+  p->ws_bytes = p->off_sync + align256(sizeof(int) * (2 + std::max(p->n, p->zcols) / 16));
   p->nz = p->n;
   return NLOS_OK;
 }
@@ -772,7 +826,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
   int* sync = reinterpret_cast<int*>(ws + p->off_sync);
   const size_t sync_bytes = sizeof(int) * (size_t)(1 + n / 16);
   const size_t cb = complex_bytes(st), rb = real_bytes(st);
-  if (p->fused) {
+  if (p->fused || p->fused_inv) {
     ch.tw = p->tw32[(int)Lx];   // radix-32 schedule
     ch.a = (int)a;
     ch.b = (int)b;
@@ -856,36 +910,58 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
   z.t_ramp = part == 2 ? ramp : 0.0f;
   z.G_n = ws_extent(p, 1);
   z.psi_n = ws_extent(p, 2);
-  z.psi_blocked = p->fused ? 1 : 0;
+  z.psi_blocked = p->fused_inv ? 1 : 0;
   z.err = err;
   if (p->zlast) {
     // FK3 without its inverses: the resampled spectra of both partners
     NLOS_CU(launch_fk_stolt(z, st, p->tiles[sid], s), "fk stolt stage");
     NLOS_MARK(p, s, sid++);
-    // FK4: y inverse (keep y < b) then x inverse (keep x < a), complex, into
-    // the second buffer (the forward spectrum is no longer needed)
-    FkChainLaunch c{};
-    c.p = ch;
-    c.p.in = b2;
-    c.p.mid = b0;
-    c.p.out = b1;
-    c.p.s1 = g2b;
-    c.p.s2 = g2a;
-    c.p.in_n = ws_extent(p, 2);
-    c.p.mid_n = ws_extent(p, 0);
-    c.p.out_n = std::min<long long>(ws_extent(p, 1), a * b * n);
-    c.p.discard = p->tiles[sid] < 2;
-    c.nslot = p->tiles[sid] % 2 == 0 ? 3 : 2;
-    c.fwd = 0;
-    c.store_mode = kStoreCpx;   // the storage type
-    NLOS_CU(cudaMemsetAsync(sync, 0, sync_bytes, s), "fk chain counters");
-    NLOS_CU(launch_fk_chain(c, st, s), "fk yx-inverse");
-    NLOS_MARK(p, s, sid++);
+    // FK4: y inverse (keep y < b) then x inverse (keep x < a), complex, over
+    // the m columns of V; buffers as fk_buffers says
+    const long long m = p->zcols;
+    const bool wide = fk_wide(p);
+    void* mid = wide ? b1 : b0;
+    void* S = wide ? b0 : b1;
+    const long long mid_n = ws_extent(p, wide ? 1 : 0), S_n = std::min<long long>(ws_extent(p, wide ? 0 : 1), a * b * m);
+    if (p->fused_inv) {
+      FkChainLaunch c{};
+      c.p = ch;
+      c.p.n = (int)m;
+      c.p.nchunks = (int)(m / 16);
+      c.p.in = b2;
+      c.p.mid = mid;
+      c.p.out = S;
+      c.p.s1 = g2b;
+      c.p.s2 = g2a;
+      c.p.in_n = ws_extent(p, 2);
+      c.p.mid_n = mid_n;
+      c.p.out_n = S_n;
+      c.p.discard = p->tiles[sid] < 2;
+      c.nslot = p->tiles[sid] % 2 == 0 ? 3 : 2;
+      c.fwd = 0;
+      c.store_mode = kStoreCpx;   // the storage type
+      NLOS_CU(cudaMemsetAsync(sync, 0, sizeof(int) * (size_t)(1 + m / 16), s), "fk chain counters");
+      NLOS_CU(launch_fk_chain(c, st, s), "fk yx-inverse");
+      NLOS_MARK(p, s, sid++);
+    } else {
+      l = axis(st, (int)Ly, Lx, b2, mid, m, Ly * m, m, b * m, m, (int)Ly, (int)b, 1, g2b, p->tw[(int)Ly], p->tiles[sid]);
+      l.err = err;
+      attach_tmap(l);
+      set_extents(l, ws_extent(p, 2), mid_n);
+      NLOS_CU(launch_axis_fft(l, s), "fk y-inverse");
+      NLOS_MARK(p, s, sid++);
+      l = axis(st, (int)Lx, 1, mid, S, b * m, 0, b * m, 0, b * m, (int)Lx, (int)a, 1, g2a, p->tw[(int)Lx], p->tiles[sid]);
+      l.err = err;
+      attach_tmap(l);
+      set_extents(l, mid_n, S_n);
+      NLOS_CU(launch_axis_fft(l, s), "fk x-inverse");
+      NLOS_MARK(p, s, sid++);
+    }
     // FK5: z inverse of the a x b kept pencils, |psi|^2 (or psi) with the normalisation
     // (the pass scales applied before this last transform now include the x inverse's)
     const double gz = gprod * g2a;
     FkZInvParams zi{};
-    zi.in = b1;
+    zi.in = S;
     zi.out = vol;
     zi.tw = p->tw[(int)Lt];
     zi.tw32 = p->tw32[(int)Lt];
@@ -895,7 +971,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
     zi.scale = (float)(cpx ? 1.0 / (N * gz) : 1.0 / (N * N * gz * gz));
     zi.dev_scale = cpx ? inv_s : inv_s2;
     zi.complex_out = cpx ? 1 : 0;
-    zi.in_n = std::min<long long>(ws_extent(p, 1), a * b * n);
+    zi.in_n = S_n;
     zi.out_n = a * b * n;
     zi.err = err;
     NLOS_CU(launch_fk_zinv(zi, st, p->tiles[sid], s), "fk z-inverse");
@@ -904,7 +980,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
   }
   NLOS_CU(launch_fk_zstage(z, st, p->tiles[sid], s), "fk stolt stage");
   NLOS_MARK(p, s, sid++);
-  if (p->fused) {
+  if (p->fused_inv) {
     // FK4 fused: y inverse (keep y < b) then x inverse (keep x < a) with |psi|^2
     FkChainLaunch c{};
     c.p = ch;
@@ -1325,21 +1401,21 @@ nlos_status_t nlos_plan_create_ex(const nlos_plan_desc_t* desc, int flags, nlos_
     p->Lt = fk ? (pad == 1 ? p->n : pow2_at_least(2 * p->n)) : pow2_at_least(p->n);
   }
   p->storage = desc->storage;
-  p->fused = desc->method == NLOS_FK && !(flags & NLOS_PLAN_SEPARATE_AXES) &&
-             fk_chain_eligible(p->a, p->b, p->n, p->Lx, p->Ly, desc->pad_factor);
-  // plans with fused lateral stages and L = 2n take the inverse temporal
-  // transform last, on the kept pencils
-  p->zlast = p->fused && p->Lt == 2 * p->n;
+  if (desc->method == NLOS_FK) fk_structure(p, flags);
   if (p->storage != kF32) p->stage_names.push_back("volume_scale");
-  const char* fk_names[] = {"fk_x_forward", "fk_y_forward", "fk_stolt_z", "fk_y_inverse", "fk_x_inverse"};
-  const char* fk_fused_names[] = {"fk_xy_forward", "fk_stolt_z", "fk_yx_inverse"};
-  const char* fk_zlast_names[] = {"fk_xy_forward", "fk_stolt", "fk_yx_inverse", "fk_z_inverse"};
   const char* pf_names[] = {"pf_band", "pf_y_forward", "pf_x_forward", "pf_depth_sum", "pf_y_inverse",
                             "pf_x_inverse"};
-  if (desc->method == NLOS_FK && p->zlast) for (const char* nm : fk_zlast_names) p->stage_names.push_back(nm);
-  else if (desc->method == NLOS_FK && p->fused) for (const char* nm : fk_fused_names) p->stage_names.push_back(nm);
-  else if (desc->method == NLOS_FK) for (const char* nm : fk_names) p->stage_names.push_back(nm);
-  else for (const char* nm : pf_names) p->stage_names.push_back(nm);
+  auto stages = [&](std::initializer_list<const char*> names) {
+    for (const char* nm : names) p->stage_names.push_back(nm);
+  };
+  if (desc->method == NLOS_FK) {
+    if (p->fused) stages({"fk_xy_forward"});
+    else stages({"fk_x_forward", "fk_y_forward"});
+    stages({p->zlast ? "fk_stolt" : "fk_stolt_z"});
+    if (p->fused_inv) stages({"fk_yx_inverse"});
+    else stages({"fk_y_inverse", "fk_x_inverse"});
+    if (p->zlast) stages({"fk_z_inverse"});
+  } else for (const char* nm : pf_names) p->stage_names.push_back(nm);
   for (const std::string& nm : p->stage_names) {
     const bool xs = nm.find("_x_") != std::string::npos, ys = nm.find("_y_") != std::string::npos;
     const bool umma = nm == "pf_depth_sum" && desc->method == NLOS_PHASOR_RSD &&
@@ -1374,9 +1450,12 @@ nlos_status_t nlos_plan_create_ex(const nlos_plan_desc_t* desc, int flags, nlos_
     if (e != cudaSuccess) st = cuda_fail(e, "workspace clear");
   }
   if (st != NLOS_OK) {
+    // device memory that does not hold this structure's buffers may hold the
+    // smaller ones'
+    const bool again = st == NLOS_ERR_OUT_OF_MEMORY && !p->injected && p->zlast && fk_wide(p);
     for (void* v : p->allocs) cudaFree(v);
     delete p;
-    return st;
+    return again ? nlos_plan_create_ex(desc, flags | kPlanSmallWorkspace, out) : st;
   }
   *out = p;
   return NLOS_OK;
@@ -1643,7 +1722,10 @@ bool g_tune_loaded = false;
 
 std::string tune_key(const nlos_plan_s* p) {
   char buf[256];
-  snprintf(buf, sizeof buf, "m%d_s%d_%dx%dx%d_F%d_D%d", p->d.method, p->storage, p->a, p->b, p->n, p->F, p->D);
+  // (the suffix keeps shapes tuned for another stage structure of the same
+  // capture apart)
+  snprintf(buf, sizeof buf, "m%d_s%d_%dx%dx%d_F%d_D%d%s", p->d.method, p->storage, p->a, p->b, p->n, p->F, p->D,
+           p->zlast && !(p->fused && !fk_wide(p)) ? (p->fused_inv ? "_zf" : "_z") : "");
   return buf;
 }
 
@@ -1720,7 +1802,9 @@ nlos_status_t nlos_plan_autotune(nlos_plan_t p, void* stream) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     tune_cache_load();
     auto it = g_tune_cache.find(key);
-    if (it != g_tune_cache.end() && it->second.size() == p->tiles.size()) {
+    bool ok = it != g_tune_cache.end() && it->second.size() == p->tiles.size();
+    for (size_t i = 0; ok && i < p->tiles.size(); ++i) ok = it->second[i] >= 0 && it->second[i] < stage_variants(p, i);
+    if (ok) {
       p->tiles = it->second;
       p->tuned = true;
       return NLOS_OK;

@@ -121,13 +121,15 @@ struct FkZParams {
 };
 cudaError_t launch_fk_zstage(const FkZParams& p, int storage, int tile, cudaStream_t s);
 
-// f-k with the inverse temporal transform last (fk_zsplit.cuh; L = 2n):
-// FK3 without its inverses (psi receives the resampled spectra V[kx][ky][m],
-// m < n) and FK5, the inverse temporal transform of the a x b kept pencils.
+// f-k with the inverse temporal transform last (fk_zsplit.cuh): FK3 without its
+// inverses (psi receives the resampled spectra V[kx][ky][m], m < L/2: the
+// strides of psi above hold with n = L/2; G keeps its n samples per pencil)
+// and FK5, the inverse temporal transform of the a x b kept pencils. L = 2n,
+// or, float32 storage only, any power of two L >= 2n.
 cudaError_t launch_fk_stolt(const FkZParams& p, int storage, int tile, cudaStream_t s);
 struct FkZInvParams {
-  const void* in;              // [npencils][n] the laterally inverted spectra (storage type), m < n = L/2
-  void* out;                   // [npencils][n] float (|.|^2) or float2 (complex_out)
+  const void* in;              // [npencils][L/2] the laterally inverted spectra (storage type), m < L/2
+  void* out;                   // [npencils][n] float (|.|^2) or float2 (complex_out), n <= L/2
   const float2* tw;            // twiddles for L
   const float2* tw32;          // twiddles of the radix-32 schedule for L
   int L, n;
@@ -173,7 +175,13 @@ struct FkChainLaunch {
   int nslot;                   // shared-memory slots per CTA (2 or 3; 2 at L = 1024)
 };
 cudaError_t launch_fk_chain(const FkChainLaunch& l, int storage, cudaStream_t s);
-// zero-padded f-k with Lx = Ly = L in [128, 1024] (at least one warp of
+// the fused inverse alone: any a, b <= L / 2 (its copies are runs of blocked
+// columns), n columns a multiple of 16
+inline bool fk_chain_inv_eligible(int n, int Lx, int Ly) { return Lx == Ly && Lx >= 128 && Lx <= 1024 && n % 16 == 0; }
+// nlos_plan_create_ex flag for the library's own callers: the temporal stage
+// with the smaller workspace where there is a choice
+constexpr int kPlanSmallWorkspace = 1 << 8;
+// the pair: zero-padded f-k with Lx = Ly = L in [128, 1024] (at least one warp of
 // transforming threads per CTA), n a multiple of 16, and every TMA box row
 // count (a, b, L) at most 256 or a multiple of it
 inline bool fk_chain_eligible(int a, int b, int n, int Lx, int Ly, int pad) {
