@@ -228,8 +228,9 @@ struct nlos_plan_s {
   std::vector<cudaEvent_t> prof_pool;
   std::vector<int> prof_stage;          // stage index of each recorded event (-1: call start)
   size_t prof_used = 0;
-  // shared-spectrum mixture of experts: spectrum ready, phasor branch done (created on first use)
-  cudaEvent_t moe_ev[2] = {nullptr, nullptr};
+  // shared-spectrum mixture of experts: spectrum ready, phasor branch done,
+  // spectrum read by the phasor branch (created on first use)
+  cudaEvent_t moe_ev[3] = {nullptr, nullptr, nullptr};
 };
 
 namespace {
@@ -792,7 +793,10 @@ void set_extents(AxisLaunch& l, long long in_n, long long out_n) {
 // without the t/(n-1) ramp (the spectrum shared with a phasor-field plan,
 // float32 plans only); 2 the rest after part 1, the ramp applied as the
 // temporal stage loads the spectrum (it commutes with the lateral transforms).
-nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStream_t s, int part) {
+// g_free (part 2, may be null): recorded on another stream that reads the
+// spectrum; waited for before the lateral inverses write over it.
+nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStream_t s, int part,
+                     cudaEvent_t g_free = nullptr) {
   const int st = p->storage;
   const long long a = p->a, b = p->b, n = p->n;
   void* b0 = ws + p->off[0];
@@ -916,6 +920,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
     // FK3 without its inverses: the resampled spectra of both partners
     NLOS_CU(launch_fk_stolt(z, st, p->tiles[sid], s), "fk stolt stage");
     NLOS_MARK(p, s, sid++);
+    if (g_free) NLOS_CU(cudaStreamWaitEvent(s, g_free, 0), "mixture-of-experts order");
     // FK4: y inverse (keep y < b) then x inverse (keep x < a), complex, over
     // the m columns of V; buffers as fk_buffers says
     const long long m = p->zcols;
@@ -1025,9 +1030,10 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
 // transform is skipped and P_in is the compact phasor field [x][y][F]; or,
 // when G0 is given (float32 plans only), the band and the lateral forward
 // transforms come from the shared spectrum G0 [Lx/2 + 1][Ly][n] (the x then y
-// forward transforms of the transient, taken once for both experts).
+// forward transforms of the transient, taken once for both experts; g_read,
+// if given, is recorded once the spectrum has been read).
 nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol, char* ws, cudaStream_t s,
-                     const void* G0) {
+                     const void* G0, cudaEvent_t g_read = nullptr) {
   const int st = p->storage;
   const long long a = p->a, b = p->b, n = p->n, F = p->F, D = p->D;
   void* b0 = ws + p->off[0];
@@ -1099,6 +1105,7 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
     sp.Phat_n = ws_extent(p, 2);
     sp.err = err;
     NLOS_CU(launch_pf_band_spectrum(sp, s), "pf band from shared spectrum");
+    if (g_read) NLOS_CU(cudaEventRecord(g_read, s), "mixture-of-experts order");
     NLOS_MARK(p, s, sid++);
     sid += 2;
   } else {
@@ -1594,7 +1601,8 @@ nlos_status_t nlos_reconstruct_moe(nlos_plan_t fk, nlos_plan_t pf, const void* t
   cudaGetLastError();
   char* wf = static_cast<char*>(fk->ws);
   // the shared spectrum lives in the f-k plan's second buffer, which the
-  // f-k temporal stage only reads and the phasor branch only reads
+  // f-k temporal stage and the phasor branch only read; the f-k lateral
+  // inverses write over it, after both
   const void* G0 = wf + fk->off[1];
   nlos_status_t st = run_fk(fk, transient, volume_fk, wf, s, 1);
   if (st != NLOS_OK) return st;
@@ -1602,9 +1610,10 @@ nlos_status_t nlos_reconstruct_moe(nlos_plan_t fk, nlos_plan_t pf, const void* t
     NLOS_CU(cudaEventRecord(fk->moe_ev[0], s), "mixture-of-experts order");
     NLOS_CU(cudaStreamWaitEvent(s2, fk->moe_ev[0], 0), "mixture-of-experts order");
   }
-  st = run_pf(pf, nullptr, nullptr, volume_pf, static_cast<char*>(pf->ws), s2, G0);
+  cudaEvent_t g_read = two ? fk->moe_ev[2] : nullptr;
+  st = run_pf(pf, nullptr, nullptr, volume_pf, static_cast<char*>(pf->ws), s2, G0, g_read);
   if (st != NLOS_OK) return st;
-  st = run_fk(fk, transient, volume_fk, wf, s, 2);
+  st = run_fk(fk, transient, volume_fk, wf, s, 2, g_read);
   if (st != NLOS_OK) return st;
   if (two) {
     // join: the next call's spectrum must not overwrite what the phasor branch still reads
