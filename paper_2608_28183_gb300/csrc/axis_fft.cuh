@@ -12,6 +12,7 @@
 #include "nlos_bounds.cuh"
 #include "nlos_fft.cuh"
 #include "nlos_internal.h"
+#include "nlos_launch.cuh"
 #include "nlos_tma.cuh"
 
 namespace nlos {
@@ -121,6 +122,8 @@ __global__ void __launch_bounds__(AxisTile<L, IC>::THREADS)
 axis_fft_realpair_kernel(const AxisParams p) {
   extern __shared__ float2 pair_sm[];
   constexpr int TPC = L / 16;
+  pdl_trigger();
+  pdl_wait();
   const int c = threadIdx.x % IC;
   const int j0 = threadIdx.x / IC;
   const long long ii0 = (long long)blockIdx.x * (2 * IC) + c;
@@ -165,14 +168,16 @@ cudaError_t launch_axis_pair_ic(const AxisLaunch& l, cudaStream_t s) {
     if (e != cudaSuccess) return e;
   }
   dim3 grid((unsigned)((l.p.inner + 2 * IC - 1) / (2 * IC)), (unsigned)l.n_outer);
-  k<<<grid, Tile::THREADS, smem, s>>>(l.p);
-  return axis_report("realpair", L, IC, Tile::THREADS, smem, grid.x, grid.y, cudaGetLastError());
+  const cudaError_t e = launch_kernel(l.after, k, grid, Tile::THREADS, smem, s, l.p);
+  return axis_report("realpair", L, IC, Tile::THREADS, smem, grid.x, grid.y, e);
 }
 
 template <int L, int IC, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut, bool INV>
 __global__ void __launch_bounds__(AxisTile<L, IC>::THREADS)
 axis_fft_kernel(const AxisParams p) {
   extern __shared__ float2 axis_sm[];
+  pdl_trigger();
+  pdl_wait();
   AxisCtx<L, IC, LD, ST, TS, INV> ctx;
   const int c = threadIdx.x % IC;
   const int j0 = threadIdx.x / IC;
@@ -253,6 +258,7 @@ axis_fft_tma_kernel(const __grid_constant__ CUtensorMap tmap, const AxisParams p
     mbar_fence_init();
   }
   __syncthreads();
+  pdl_wait();
   auto issue = [&](long long tile, int slot) {
     const int ti = (int)(tile % tiles_inner);
     const int to = (int)(tile / tiles_inner);
@@ -270,6 +276,7 @@ axis_fft_tma_kernel(const __grid_constant__ CUtensorMap tmap, const AxisParams p
     const int slot = k & 1;
     const long long next = tile + gridDim.x;
     if (threadIdx.x == 0 && next < ntiles) issue(next, slot ^ 1);
+    if (next >= ntiles) pdl_trigger();
     if (!mbar_wait_bounded(&bar[slot], (k >> 1) & 1, kTmaWaitLimit)) {
       if (err) atomicExch(err, kDevErrTmaTimeout);
       // give the copies still in flight into this CTA's buffers a last
@@ -326,8 +333,9 @@ cudaError_t launch_axis_tma(const AxisLaunch& l, cudaStream_t s) {
   const int tiles_inner = (int)((l.p.inner + IC - 1) / IC);
   const long long ntiles = (long long)tiles_inner * l.n_outer;
   const long long grid = std::min<long long>(ntiles, (long long)sms * blocks_per_sm);
-  k<<<(unsigned)grid, T::THREADS, T::SMEM, s>>>(l.tmap, l.p, tiles_inner, ntiles, l.err);
-  return axis_report("tma", L, IC, T::THREADS, T::SMEM, grid, ntiles, cudaGetLastError());
+  const cudaError_t e =
+      launch_kernel(l.after, k, dim3((unsigned)grid), T::THREADS, T::SMEM, s, l.tmap, l.p, tiles_inner, ntiles, l.err);
+  return axis_report("tma", L, IC, T::THREADS, T::SMEM, grid, ntiles, e);
 }
 
 // ---------------------------------------------------------------------------
@@ -376,6 +384,7 @@ axis_fft_tma_pair_kernel(const __grid_constant__ CUtensorMap tmap, const AxisPar
     mbar_fence_init();
   }
   __syncthreads();
+  pdl_wait();
   auto issue = [&](long long tile, int slot) {
     const int ti = (int)(tile % tiles_inner);
     const int to = (int)(tile / tiles_inner);
@@ -394,6 +403,7 @@ axis_fft_tma_pair_kernel(const __grid_constant__ CUtensorMap tmap, const AxisPar
     const int slot = k & 1;
     const long long next = tile + gridDim.x;
     if (threadIdx.x == 0 && next < ntiles) issue(next, slot ^ 1);
+    if (next >= ntiles) pdl_trigger();
     if (!mbar_wait_bounded(&bar[slot], (k >> 1) & 1, kTmaWaitLimit)) {
       if (err) atomicExch(err, kDevErrTmaTimeout);
       // give the copies still in flight into this CTA's buffers a last
@@ -450,8 +460,9 @@ cudaError_t launch_axis_tma_pair(const AxisLaunch& l, cudaStream_t s) {
   const int tiles_inner = (int)((l.p.inner + 2 * IC - 1) / (2 * IC));
   const long long ntiles = (long long)tiles_inner * l.n_outer;
   const long long grid = std::min<long long>(ntiles, (long long)sms * blocks_per_sm);
-  k<<<(unsigned)grid, THREADS, SMEM, s>>>(l.tmap, l.p, tiles_inner, ntiles, l.err);
-  return axis_report("tma-pair", L, IC, THREADS, SMEM, grid, ntiles, cudaGetLastError());
+  const cudaError_t e =
+      launch_kernel(l.after, k, dim3((unsigned)grid), THREADS, SMEM, s, l.tmap, l.p, tiles_inner, ntiles, l.err);
+  return axis_report("tma-pair", L, IC, THREADS, SMEM, grid, ntiles, e);
 }
 
 // real-pair variants: tiles [0, n) direct loads, [2n, 3n) TMA staging (n
@@ -481,8 +492,8 @@ cudaError_t launch_axis_ic(const AxisLaunch& l, cudaStream_t s) {
     if (e != cudaSuccess) return e;
   }
   dim3 grid((unsigned)((l.p.inner + Tile::IC - 1) / Tile::IC), (unsigned)l.n_outer);
-  k<<<grid, Tile::THREADS, Tile::SMEM, s>>>(l.p);
-  return axis_report("direct", L, IC, Tile::THREADS, Tile::SMEM, grid.x, grid.y, cudaGetLastError());
+  const cudaError_t e = launch_kernel(l.after, k, grid, Tile::THREADS, Tile::SMEM, s, l.p);
+  return axis_report("direct", L, IC, Tile::THREADS, Tile::SMEM, grid.x, grid.y, e);
 }
 
 template <int L, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut, bool INV>

@@ -226,6 +226,7 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map, const FkChainParams p) 
   }
   for (int i = threadIdx.x; i < FftShape<L, kChainE>::TWSIZE; i += T::THREADS) tw[i] = __ldg(p.tw + i);
   __syncthreads();
+  pdl_wait();
 
   if (threadIdx.x >= T::CONSUMERS) {
     // ------------------------------ producer ------------------------------
@@ -252,6 +253,7 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map, const FkChainParams p) 
       if (t >= total) {
         d.state = 1;
         mbar_arrive(&full[slot]);
+        pdl_trigger();
         return;
       }
       const ChainItem it = chain_decode(t, n1, n2, p.nchunks, p.lag);
@@ -443,8 +445,7 @@ cudaError_t launch_fk_chain_one(const FkChainLaunch& l, cudaStream_t s) {
   FkChainParams q = p;
   q.lag = 1 + (grid + per_chunk - 1) / per_chunk;
   if (q.lag > q.nchunks) q.lag = q.nchunks;
-  k<<<grid, T::THREADS, T::SMEM, s>>>(l.map, q);
-  return cudaGetLastError();
+  return launch_kernel(l.after, k, dim3((unsigned)grid), T::THREADS, T::SMEM, s, l.map, q);
 }
 
 // Each translation unit instantiates one storage type.

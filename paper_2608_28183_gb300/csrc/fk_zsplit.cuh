@@ -32,6 +32,7 @@
 #include "nlos_bounds.cuh"
 #include "nlos_fft.cuh"
 #include "nlos_internal.h"
+#include "nlos_launch.cuh"
 
 namespace nlos {
 
@@ -97,6 +98,8 @@ template <int L, int PPC, class TS, bool kRamp, bool kGuard, int E>
 __global__ void __launch_bounds__(FkLiteTile<L, PPC, E>::THREADS, FkLiteTile<L, PPC, E>::MINB) fk_stolt_kernel(const FkZParams p) {
   using S = FftShape<L, E>;
   extern __shared__ float2 fl_sm[];
+  pdl_trigger();
+  pdl_wait();
   const int w = threadIdx.x / S::TPC;
   const int j0 = threadIdx.x % S::TPC;
   constexpr bool kPlaces = sizeof(TS) == 8;   // psi_pos order of the blocked layout
@@ -225,6 +228,8 @@ template <int L, int PPC, class TS, bool kCpx, bool kGuard, int E>
 __global__ void __launch_bounds__(FkLiteTile<L, PPC, E>::THREADS, FkLiteTile<L, PPC, E>::MINB) fk_zinv_kernel(const FkZInvParams p) {
   using S = FftShape<L, E>;
   extern __shared__ float2 zi_sm[];
+  pdl_trigger();
+  pdl_wait();
   const int w = threadIdx.x / S::TPC;
   const int j0 = threadIdx.x % S::TPC;
   const long long pid = (long long)blockIdx.x * PPC + w;
@@ -249,8 +254,7 @@ cudaError_t launch_fk_stolt_as(const FkZParams& p, cudaStream_t s) {
     if (e != cudaSuccess) return e;
   }
   const long long blocks = (p.npencils + PPC - 1) / PPC;
-  k<<<(unsigned)blocks, T::THREADS, T::SMEM, s>>>(p);
-  return cudaGetLastError();
+  return launch_kernel(p.after, k, dim3((unsigned)blocks), T::THREADS, T::SMEM, s, p);
 }
 
 // L > 2n: float32 storage only
@@ -270,8 +274,7 @@ cudaError_t launch_fk_zinv_as(const FkZInvParams& p, cudaStream_t s) {
     if (e != cudaSuccess) return e;
   }
   const long long blocks = (p.npencils + PPC - 1) / PPC;
-  k<<<(unsigned)blocks, T::THREADS, T::SMEM, s>>>(p);
-  return cudaGetLastError();
+  return launch_kernel(p.after, k, dim3((unsigned)blocks), T::THREADS, T::SMEM, s, p);
 }
 
 template <int L, int PPC, class TS, bool kCpx, int E = 16>

@@ -25,6 +25,7 @@
 #include "nlos_bounds.cuh"
 #include "nlos_fft.cuh"
 #include "nlos_internal.h"
+#include "nlos_launch.cuh"
 
 namespace nlos {
 
@@ -134,6 +135,8 @@ __global__ void __launch_bounds__(FkTile<L, PPC, kAlias>::THREADS, FkTile<L, PPC
 fk_zstage_kernel(const FkZParams p) {
   using S = FftShape<L>;
   extern __shared__ float2 fk_sm[];
+  pdl_trigger();
+  pdl_wait();
   const int w = threadIdx.x / S::TPC;
   const int j0 = threadIdx.x % S::TPC;
   const long long pid = (long long)blockIdx.x * PPC + w;
@@ -178,8 +181,7 @@ cudaError_t launch_fk_ppc(const FkZParams& p, cudaStream_t s) {
     if (e != cudaSuccess) return e;
   }
   const long long blocks = (p.npencils + T::PPC - 1) / T::PPC;
-  k<<<(unsigned)blocks, T::THREADS, T::SMEM, s>>>(p);
-  return cudaGetLastError();
+  return launch_kernel(p.after, k, dim3((unsigned)blocks), T::THREADS, T::SMEM, s, p);
 }
 
 // tiles 0/1: the two CTA sizes; 2/3: the same with aliased buffers

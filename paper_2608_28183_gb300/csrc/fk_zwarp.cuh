@@ -26,6 +26,7 @@
 #include "nlos_bounds.cuh"
 #include "nlos_fft.cuh"
 #include "nlos_internal.h"
+#include "nlos_launch.cuh"
 
 namespace nlos {
 
@@ -113,6 +114,8 @@ template <int L, class TS, bool kPad2, bool kGuard>
 __global__ void __launch_bounds__(64) fk_zwarp_kernel(const FkZParams p) {
   using Sh = FkWarpShape<L>;
   extern __shared__ float2 zw_sm[];
+  pdl_trigger();
+  pdl_wait();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float2* U = zw_sm + w * Sh::BUF;
   float2* W = zw_sm + (2 + w) * Sh::BUF;
@@ -185,8 +188,7 @@ cudaError_t launch_fk_warp(const FkZParams& p, cudaStream_t s) {
     if (e != cudaSuccess) return e;
   }
   const long long units = (long long)(p.a_pad / 2 + 1) * (p.b_pad / 2 + 1);
-  k<<<(unsigned)units, 64, Sh::SMEM, s>>>(p);
-  return cudaGetLastError();
+  return launch_kernel(p.after, k, dim3((unsigned)units), 64, Sh::SMEM, s, p);
 }
 
 }  // namespace nlos

@@ -827,9 +827,16 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
   const bool cpx = p->d.output == NLOS_OUT_COMPLEX;
   const float fscale = (float)(cpx ? 1.0 / (N * gprod) : 1.0 / (N * N * gprod * gprod));
   FkChainParams ch{};
+  // chunk counters of the fused forward at off_sync, those of the fused inverse
+  // in the 256-byte steps before it (the scale partials' end, free once the
+  // volume scale is known): one clear for both, ahead of the first stage
   int* sync = reinterpret_cast<int*>(ws + p->off_sync);
-  const size_t sync_bytes = sizeof(int) * (size_t)(1 + n / 16);
-  const size_t cb = complex_bytes(st), rb = real_bytes(st);
+  const size_t inv_sync_bytes = p->fused_inv ? align256(sizeof(int) * (size_t)(1 + p->zcols / 16)) : 0;
+  int* sync_inv = reinterpret_cast<int*>(ws + p->off_sync - inv_sync_bytes);
+  const size_t sync_bytes = inv_sync_bytes + (p->fused ? sizeof(int) * (size_t)(1 + n / 16) : 0);
+  const size_t rb = real_bytes(st);
+  bool after = false;   // another kernel of this call precedes
+  if (part != 2 && sync_bytes) NLOS_CU(cudaMemsetAsync(sync_inv, 0, sync_bytes, s), "fk chain counters");
   if (p->fused || p->fused_inv) {
     ch.tw = p->tw32[(int)Lx];   // radix-32 schedule
     ch.a = (int)a;
@@ -867,8 +874,8 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
     if (!encode_3d(&c.map, H, rb, (unsigned long long)(b * n), a, 1, b * n * rb, a * b * n * rb, 16,
                    (unsigned)std::min<long long>(a, 256), false))
       return fail(NLOS_ERR_CUDA, "fk xy-forward: tensor map encoding failed");
-    NLOS_CU(cudaMemsetAsync(sync, 0, sync_bytes, s), "fk chain counters");
     NLOS_CU(launch_fk_chain(c, st, s), "fk xy-forward");
+    after = true;
     NLOS_MARK(p, s, sid++);
   } else {
   // FK1: x forward (real input, scaled by t/(n-1), zero-padded to Lx, kx in [0, Lx/2])
@@ -885,12 +892,14 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
   attach_tmap(l);
   set_extents(l, a * b * n, ws_extent(p, 0));
   NLOS_CU(launch_axis_fft(l, s), "fk x-forward");
+  after = true;
   NLOS_MARK(p, s, sid++);
   // FK1: y forward (zero-padded to Ly)
   l = axis(st, (int)Ly, hx, b0, b1, n, b * n, n, Ly * n, n, (int)b, (int)Ly, 0, g2b, p->tw[(int)Ly], p->tiles[sid]);
   l.err = err;
   attach_tmap(l);
   set_extents(l, ws_extent(p, 0), ws_extent(p, 1));
+  l.after = after;
   NLOS_CU(launch_axis_fft(l, s), "fk y-forward");
   NLOS_MARK(p, s, sid++);
   }
@@ -916,6 +925,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
   z.psi_n = ws_extent(p, 2);
   z.psi_blocked = p->fused_inv ? 1 : 0;
   z.err = err;
+  z.after = after;
   if (p->zlast) {
     // FK3 without its inverses: the resampled spectra of both partners
     NLOS_CU(launch_fk_stolt(z, st, p->tiles[sid], s), "fk stolt stage");
@@ -945,7 +955,8 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
       c.nslot = p->tiles[sid] % 2 == 0 ? 3 : 2;
       c.fwd = 0;
       c.store_mode = kStoreCpx;   // the storage type
-      NLOS_CU(cudaMemsetAsync(sync, 0, sizeof(int) * (size_t)(1 + m / 16), s), "fk chain counters");
+      c.p.sync = sync_inv;
+      c.after = !g_free;
       NLOS_CU(launch_fk_chain(c, st, s), "fk yx-inverse");
       NLOS_MARK(p, s, sid++);
     } else {
@@ -953,12 +964,14 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
       l.err = err;
       attach_tmap(l);
       set_extents(l, ws_extent(p, 2), mid_n);
+      l.after = !g_free;
       NLOS_CU(launch_axis_fft(l, s), "fk y-inverse");
       NLOS_MARK(p, s, sid++);
       l = axis(st, (int)Lx, 1, mid, S, b * m, 0, b * m, 0, b * m, (int)Lx, (int)a, 1, g2a, p->tw[(int)Lx], p->tiles[sid]);
       l.err = err;
       attach_tmap(l);
       set_extents(l, mid_n, S_n);
+      l.after = true;
       NLOS_CU(launch_axis_fft(l, s), "fk x-inverse");
       NLOS_MARK(p, s, sid++);
     }
@@ -979,6 +992,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
     zi.in_n = S_n;
     zi.out_n = a * b * n;
     zi.err = err;
+    zi.after = true;
     NLOS_CU(launch_fk_zinv(zi, st, p->tiles[sid], s), "fk z-inverse");
     NLOS_MARK(p, s, sid++);
     return NLOS_OK;
@@ -1002,7 +1016,8 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
     c.nslot = p->tiles[sid] % 2 == 0 ? 3 : 2;
     c.fwd = 0;
     c.store_mode = cpx ? kStoreCpx32 : kStoreAbs2;
-    NLOS_CU(cudaMemsetAsync(sync, 0, sync_bytes, s), "fk chain counters");
+    c.p.sync = sync_inv;
+    c.after = true;
     NLOS_CU(launch_fk_chain(c, st, s), "fk yx-inverse");
     NLOS_MARK(p, s, sid++);
     return NLOS_OK;
@@ -1012,6 +1027,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
   l.err = err;
   attach_tmap(l);
   set_extents(l, ws_extent(p, 2), ws_extent(p, 0));
+  l.after = true;
   NLOS_CU(launch_axis_fft(l, s), "fk y-inverse");
   NLOS_MARK(p, s, sid++);
   // FK4: x inverse (keep x < a), |psi|^2 with the 1/(Lx Ly Lt) normalisation
@@ -1021,6 +1037,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
   l.err = err;
   attach_tmap(l);
   set_extents(l, ws_extent(p, 0), a * b * n);
+  l.after = true;
   NLOS_CU(launch_axis_fft(l, s), "fk x-inverse");
   NLOS_MARK(p, s, sid++);
   return NLOS_OK;
@@ -1109,6 +1126,7 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
     NLOS_MARK(p, s, sid++);
     sid += 2;
   } else {
+  bp.after = st != kF32;   // the volume scale's kernel precedes it, with no memset between
   if (!P_in) NLOS_CU(launch_pf_band(bp, st, s), "pf band transform");
   NLOS_MARK(p, s, sid++);
   // PF2: top-left padding and 2D forward transform (y then x) of every band slice
@@ -1116,18 +1134,20 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
   l.err = err;
   attach_tmap(l);
   set_extents(l, P_in ? a * b * F : ws_extent(p, 0), ws_extent(p, 1));
+  l.after = !P_in;
   NLOS_CU(launch_axis_fft(l, s), "pf y-forward");
   NLOS_MARK(p, s, sid++);
   l = axis(st, (int)Nu, 1, b1, b2, Nv * F, 0, Nv * F, 0, Nv * F, (int)a, (int)Nu, 0, g2a, p->tw[(int)Nu], p->tiles[sid]);
   l.err = err;
   attach_tmap(l);
   set_extents(l, ws_extent(p, 1), ws_extent(p, 2));
+  l.after = true;
   NLOS_CU(launch_axis_fft(l, s), "pf x-forward");
   NLOS_MARK(p, s, sid++);
   }
   if (p->d.method == NLOS_PHASOR_DENSE) {
     // PF3, dense kernel: C = sum_f Phat * Khat (Alg. 3), every pixel written
-    PfDenseParams dp{static_cast<const float2*>(b2), p->Kd, static_cast<float2*>(b1), Nu * Nv, (int)F, (int)D};
+    PfDenseParams dp{!g_read, static_cast<const float2*>(b2), p->Kd, static_cast<float2*>(b1), Nu * Nv, (int)F, (int)D};
     NLOS_CU(launch_pf_dense(dp, s), "pf dense depth sum");
   } else {
     // PF3: depth sum (pixels beyond the cutoff stay zero); f16 and float32
@@ -1136,6 +1156,8 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
     // rows the depth sum does not store: pixels beyond the cutoff, and the
     // rows of tiles whose frequency sum is split (their parts are added)
     const size_t row_bytes = complex_bytes(st) * D;
+    // a kernel of this call precedes, unless an event or a memset lies between
+    bool depth_after = !g_read;
     if (p->Bu && p->tiles[sid] != 1) {
       PfUmmaParams up{};
       up.Phat = b2;
@@ -1160,6 +1182,7 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
         if (P_in) {
           NLOS_CU(cudaMemsetAsync(amax, 0, sizeof(unsigned), s), "phasor bound clear");
           NLOS_CU(launch_absmax(static_cast<const float*>(P), 2 * a * b * F, amax, s), "phasor bound");
+          depth_after = false;   // (absmax was launched plainly)
         }
         // (phasors taken from the shared spectrum had their own maximum recorded)
         int e2 = 0;
@@ -1174,12 +1197,14 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
       const bool ws_sched = p->tiles[sid] != 2;
       const int t0 = ws_sched ? pf_umma_first_split_tile(up) : up.ntiles;
       NLOS_CU(launch_clear_rows2(b1, p->clr_pix, p->nclr, p->tu_pix + (size_t)t0 * kUmmaTile,
-                                 (long long)(up.ntiles - t0) * kUmmaTile, row_bytes, s),
+                                 (long long)(up.ntiles - t0) * kUmmaTile, row_bytes, depth_after, s),
               "pf clear");
+      up.after = depth_after || p->nclr > 0 || t0 < up.ntiles;
       NLOS_CU(launch_pf_umma(up, ws_sched, s), "pf depth sum (tensor cores)");
     } else {
-    NLOS_CU(launch_clear_rows(b1, p->clr_pix, p->nclr, row_bytes, s), "pf clear");
+    NLOS_CU(launch_clear_rows(b1, p->clr_pix, p->nclr, row_bytes, depth_after, s), "pf clear");
     PfDepthParams dp{};
+    dp.after = depth_after || p->nclr > 0;
     dp.Phat = b2;
     dp.K = p->Kr;
     dp.C = b1;
@@ -1200,6 +1225,7 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
   l.err = err;
   attach_tmap(l);
   set_extents(l, ws_extent(p, 1), ws_extent(p, 0));
+  l.after = true;
   NLOS_CU(launch_axis_fft(l, s), "pf y-inverse");
   NLOS_MARK(p, s, sid++);
   // scales the data carries into this last pass (it applies none of its own)
@@ -1211,6 +1237,7 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
   l.err = err;
   attach_tmap(l);
   set_extents(l, ws_extent(p, 0), a * b * D);
+  l.after = true;
   NLOS_CU(launch_axis_fft(l, s), "pf x-inverse");
   NLOS_MARK(p, s, sid++);
   return NLOS_OK;
@@ -1546,6 +1573,7 @@ nlos_status_t nlos_bin_phasors(nlos_plan_t p, const uint32_t* pixel, const uint3
     bp.ld_scale = 1.0f;
     bp.st_scale = 1.0f;
     bp.accumulate = accumulate ? 1 : 0;
+    bp.after = false;
     NLOS_CU(launch_pf_band(bp, kF32, s), "phasors from histogram");
     return NLOS_OK;
   }
@@ -1836,13 +1864,24 @@ nlos_status_t nlos_plan_autotune(nlos_plan_t p, void* stream) {
     nlos_status_t r = run_plan(p, din, dout, ws, s);
     if (r != NLOS_OK) return r;
     NLOS_CU(cudaEventRecord(e0, s), "autotune timing");
-    for (int k = 0; k < 3; ++k) {
-      r = run_plan(p, din, dout, ws, s);
-      if (r != NLOS_OK) return r;
+    // at least three runs, and about a millisecond: the variants of a short
+    // sequence differ by less than three runs of it resolve
+    int runs = 0;
+    for (int want = 3; runs < want;) {
+      for (; runs < want; ++runs) {
+        r = run_plan(p, din, dout, ws, s);
+        if (r != NLOS_OK) return r;
+      }
+      NLOS_CU(cudaEventRecord(e1, s), "autotune timing");
+      NLOS_CU(cudaEventSynchronize(e1), "autotune timing");
+      NLOS_CU(cudaEventElapsedTime(ms, e0, e1), "autotune timing");
+      if (want > 3 || *ms >= 1.0f) break;
+      want = std::min(24, (int)(3.0f / std::max(*ms, 0.01f)));
+      if (want <= 3) break;
+      runs = 0;
+      NLOS_CU(cudaEventRecord(e0, s), "autotune timing");
     }
-    NLOS_CU(cudaEventRecord(e1, s), "autotune timing");
-    NLOS_CU(cudaEventSynchronize(e1), "autotune timing");
-    NLOS_CU(cudaEventElapsedTime(ms, e0, e1), "autotune timing");
+    *ms /= (float)runs;
     return NLOS_OK;
   };
   for (size_t i = 0; st == NLOS_OK && i < p->tiles.size(); ++i) {

@@ -40,6 +40,7 @@ struct AxisParams {
 
 struct AxisLaunch {
   AxisParams p;
+  bool after;                  // launched after another kernel of the same call (nlos_launch.cuh)
   int tile;                    // launch-shape variant: column tile = tile % n, TMA staging = tile / n
   CUtensorMap tmap;            // input tensor map for TMA staging (valid if has_tmap)
   int has_tmap;
@@ -99,6 +100,7 @@ __host__ __device__ constexpr int psi_pos(int ky, int h) {
 // fused lateral inverse: [kx'][z / 8][place of ky'][z % 8], where the place is
 // psi_pos(ky', b_pad / 2) for float32 storage and ky' for 16-bit storage.
 struct FkZParams {
+  bool after;                  // launched after another kernel of the same call (nlos_launch.cuh)
   const void* G;
   void* psi;
   const float2* tw;            // twiddles for the temporal length L
@@ -128,6 +130,7 @@ cudaError_t launch_fk_zstage(const FkZParams& p, int storage, int tile, cudaStre
 // or, float32 storage only, any power of two L >= 2n.
 cudaError_t launch_fk_stolt(const FkZParams& p, int storage, int tile, cudaStream_t s);
 struct FkZInvParams {
+  bool after;                  // launched after another kernel of the same call (nlos_launch.cuh)
   const void* in;              // [npencils][L/2] the laterally inverted spectra (storage type), m < L/2
   void* out;                   // [npencils][n] float (|.|^2) or float2 (complex_out), n <= L/2
   const float2* tw;            // twiddles for L
@@ -169,6 +172,7 @@ struct FkChainParams {
 };
 struct FkChainLaunch {
   FkChainParams p;
+  bool after;                  // launched after another kernel of the same call (nlos_launch.cuh)
   CUtensorMap map;             // forward: TMA map of the transient
   int fwd;                     // 1 forward, 0 inverse
   int store_mode;              // inverse: kStoreAbs2 or kStoreCpx32
@@ -193,6 +197,7 @@ inline bool fk_chain_eligible(int a, int b, int n, int Lx, int Ly, int pad) {
 // Phasor-field temporal band transform: per wall pencil H[x][y][0..n) (real),
 // length-n DFT, keep bins k_lo..k_lo+F-1, multiply by w(f): P[x][y][f].
 struct PfBandParams {
+  bool after;                  // launched after another kernel of the same call (nlos_launch.cuh)
   const void* H;
   void* P;
   const float2* tw;            // twiddles for L
@@ -253,6 +258,7 @@ cudaError_t launch_bin_transient(const uint32_t* pixel, const uint32_t* ticks, l
 // C[pix][d] = acut * sum_f Phat[pix][f] * ((1 - alpha) K[i0][f][d] + alpha K[i1][f][d]).
 constexpr int kPfChunk = 16;
 struct PfDepthParams {
+  bool after;                  // launched after another kernel of the same call (nlos_launch.cuh)
   const void* Phat;            // [Nu*Nv][F] complex (storage type)
   const void* K;               // [N_rho][F][D] complex (kernel storage type)
   void* C;                     // [Nu*Nv][D] complex (storage type)
@@ -303,6 +309,7 @@ __host__ __device__ constexpr int umma_row_bytes(int) { return 64; }
 __host__ __device__ constexpr int umma_chunk_cols(int) { return 32; }
 __host__ __device__ constexpr int umma_parts(int kind) { return kind == kUmmaF16 ? 1 : 2; }
 struct PfUmmaParams {
+  bool after;                  // launched after another kernel of the same call (nlos_launch.cuh)
   const void* Phat;            // [npix][F] half2 (f16 kind) or float2 (f16x3 kind)
   const void* B;               // [n_rho][nblk][KC][parts][2 Db rows x row bytes], operand layout
   void* C;                     // [npix][D] half2 or float2
@@ -329,10 +336,10 @@ cudaError_t launch_pf_umma(const PfUmmaParams& p, bool pipelined, cudaStream_t s
 int pf_umma_first_split_tile(const PfUmmaParams& p);
 // zero `row_bytes` (a multiple of 4) at C + pix * row_bytes for every
 // pix = list[i] >= 0, i < n
-cudaError_t launch_clear_rows(void* C, const int* list, long long n, size_t row_bytes, cudaStream_t s);
+cudaError_t launch_clear_rows(void* C, const int* list, long long n, size_t row_bytes, bool after, cudaStream_t s);
 // the same for the entries of two lists in one launch
 cudaError_t launch_clear_rows2(void* C, const int* l1, long long n1, const int* l2, long long n2, size_t row_bytes,
-                               cudaStream_t s);
+                               bool after, cudaStream_t s);
 // max |x| over `count` floats into *out (float bits, atomicMax; *out must be
 // cleared beforehand)
 cudaError_t launch_absmax(const float* x, long long count, unsigned* out, cudaStream_t s);
@@ -353,6 +360,7 @@ struct DenseGenParams {
 cudaError_t launch_dense_gen(const DenseGenParams& p, cudaStream_t s);
 // Dense depth sum: C[pix][d] = sum_f Phat[pix][f] * Khat[pix][f][d] (float32).
 struct PfDenseParams {
+  bool after;                  // launched after another kernel of the same call (nlos_launch.cuh)
   const float2* Phat;          // [npix][F]
   const float2* K;             // [npix][F][D]
   float2* C;                   // [npix][D]

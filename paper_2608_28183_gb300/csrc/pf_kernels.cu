@@ -4,6 +4,7 @@
 #include "nlos_bounds.cuh"
 #include "nlos_fft.cuh"
 #include "nlos_internal.h"
+#include "nlos_launch.cuh"
 #include "nlos_tma.cuh"
 #include "nlos_umma.cuh"
 
@@ -116,6 +117,8 @@ pf_band_kernel(const PfBandParams p) {
   using S = FftShape<L>;
   using T = PfBandTile<L>;
   extern __shared__ __align__(16) unsigned char pfb_sm[];
+  pdl_trigger();
+  pdl_wait();
   const int w = threadIdx.x / S::TPC;
   const int j0 = threadIdx.x % S::TPC;
   const long long q0 = 2 * ((long long)blockIdx.x * T::PPC + w);    // the pair's first pencil
@@ -154,6 +157,7 @@ pf_band_staged_kernel(const PfBandParams p, const long long nsets) {
     mbar_fence_init();
   }
   __syncthreads();
+  pdl_wait();
   const TR* H = static_cast<const TR*>(p.H);
   auto issue = [&](long long set, int slot) {
     const long long first = 2 * T::PPC * set;
@@ -173,6 +177,7 @@ pf_band_staged_kernel(const PfBandParams p, const long long nsets) {
     const int slot = k & 1;
     const long long next = set + gridDim.x;
     if (threadIdx.x == 0 && next < nsets) issue(next, slot ^ 1);
+    if (next >= nsets) pdl_trigger();
     // every thread waits for the slot; a wait that gives up anywhere sends
     // the whole CTA out (after a last bounded wait for its copies in flight)
     const bool ok = __syncthreads_and(mbar_wait_bounded(&bar[slot], (k >> 1) & 1, kBandWaitLimit));
@@ -229,8 +234,7 @@ static cudaError_t launch_band_one(const PfBandParams& p, cudaStream_t s) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, T::THREADS, smem);
     if (e != cudaSuccess) return e;
     const long long grid = std::min<long long>(nsets, (long long)band_sm_count() * std::max(per, 1));
-    k<<<(unsigned)grid, T::THREADS, smem, s>>>(p, nsets);
-    return cudaGetLastError();
+    return launch_kernel(p.after, k, dim3((unsigned)grid), T::THREADS, smem, s, p, nsets);
   }
   auto k = pf_band_kernel<L, TR, TS>;
   const size_t smem = T::smem(p.F, false);
@@ -238,8 +242,7 @@ static cudaError_t launch_band_one(const PfBandParams& p, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k<<<(unsigned)nsets, T::THREADS, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_kernel(p.after, k, dim3((unsigned)nsets), T::THREADS, smem, s, p);
 }
 
 template <class TR, class TS>
@@ -317,6 +320,7 @@ pf_band_spectrum_kernel(const PfSpecParams p) {
   using S = FftShape<L>;
   constexpr int PPC = PfBandTile<L>::PPC;
   extern __shared__ float2 pfs_sm[];
+  pdl_trigger();
   const int w = threadIdx.x / S::TPC;
   const int j0 = threadIdx.x % S::TPC;
   const long long np = (long long)(p.Lx / 2 + 1) * p.Ly;
@@ -393,6 +397,8 @@ pf_depth_kernel(const PfDepthParams p) {
   extern __shared__ float4 ps4[];   // [F][kPfChunk / 2] pairs of the chunk's phasors
   __shared__ int pix[kPfChunk];
   __shared__ float sal[kPfChunk], sac[kPfChunk];
+  pdl_trigger();
+  pdl_wait();
   const int ch = blockIdx.x;
   const int d0 = blockIdx.y * kDepthBlock + threadIdx.x;
   if (threadIdx.x < kPfChunk) {
@@ -476,8 +482,7 @@ static cudaError_t launch_depth_typed(const PfDepthParams& p, cudaStream_t s) {
     if (e != cudaSuccess) return e;
   }
   dim3 grid((unsigned)p.nchunks, (unsigned)((p.D + kDepthBlock - 1) / kDepthBlock));
-  k<<<grid, kDepthThreads, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_kernel(p.after, k, grid, kDepthThreads, smem, s, p);
 }
 
 cudaError_t launch_pf_depth(const PfDepthParams& p, int storage, int kstorage, cudaStream_t s) {
@@ -647,6 +652,7 @@ __global__ void sumsq_partial_kernel(const TR* H, long long count, int n, float 
   __shared__ float red[256];
   __shared__ double dred[256];
   __shared__ bool last;
+  pdl_trigger();
   float acc = 0.f;
   const long long chunks = count / 8;
   const long long q0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -777,6 +783,8 @@ cudaError_t launch_dense_gen(const DenseGenParams& p, cudaStream_t s) {
 // evict first), four frequencies in flight.
 __global__ void __launch_bounds__(128) pf_dense_kernel(const PfDenseParams p) {
   extern __shared__ float2 ph_sm[];
+  pdl_trigger();
+  pdl_wait();
   const long long pix = blockIdx.x;
   for (int f = threadIdx.x; f < p.F; f += blockDim.x) ph_sm[f] = p.Phat[pix * p.F + f];
   __syncthreads();
@@ -808,6 +816,7 @@ __global__ void __launch_bounds__(128) pf_dense_kernel(const PfDenseParams p) {
 // 16-byte aligned (a scalar tail covers the rest), warp maximum, one atomicMax
 // of the float bits per warp (bits of non-negative floats order like the values)
 __global__ void absmax_kernel(const float* x, long long count, bool aligned, unsigned* out) {
+  pdl_trigger();
   float m = 0.f;
   const long long n4 = aligned ? count / 4 : 0;
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -836,6 +845,8 @@ cudaError_t launch_absmax(const float* x, long long count, unsigned* out, cudaSt
 // one warp per listed row (first list, then second): 4-byte stores across the lanes
 __global__ void clear_rows2_kernel(unsigned* C, const int* l1, long long n1, const int* l2, long long n2,
                                    long long row_words) {
+  pdl_trigger();
+  pdl_wait();
   const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= n1 + n2) return;
@@ -846,18 +857,17 @@ __global__ void clear_rows2_kernel(unsigned* C, const int* l1, long long n1, con
 }
 
 cudaError_t launch_clear_rows2(void* C, const int* l1, long long n1, const int* l2, long long n2, size_t row_bytes,
-                               cudaStream_t s) {
+                               bool after, cudaStream_t s) {
   if (n1 < 0 || n2 < 0) return cudaErrorInvalidValue;
   if (n1 + n2 == 0) return cudaSuccess;
   if (!C || (n1 && !l1) || (n2 && !l2) || row_bytes % 4) return cudaErrorInvalidValue;
   const long long threads = (n1 + n2) * 32;
-  clear_rows2_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(static_cast<unsigned*>(C), l1, n1, l2, n2,
-                                                                      (long long)(row_bytes / 4));
-  return cudaGetLastError();
+  return launch_kernel(after, clear_rows2_kernel, dim3((unsigned)((threads + 255) / 256)), 256, 0, s,
+                       static_cast<unsigned*>(C), l1, n1, l2, n2, (long long)(row_bytes / 4));
 }
 
-cudaError_t launch_clear_rows(void* C, const int* list, long long n, size_t row_bytes, cudaStream_t s) {
-  return launch_clear_rows2(C, list, n, nullptr, 0, row_bytes, s);
+cudaError_t launch_clear_rows(void* C, const int* list, long long n, size_t row_bytes, bool after, cudaStream_t s) {
+  return launch_clear_rows2(C, list, n, nullptr, 0, row_bytes, after, s);
 }
 
 cudaError_t launch_pf_dense(const PfDenseParams& p, cudaStream_t s) {
@@ -868,8 +878,7 @@ cudaError_t launch_pf_dense(const PfDenseParams& p, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(pf_dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  pf_dense_kernel<<<(unsigned)p.npix, threads, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_kernel(p.after, pf_dense_kernel, dim3((unsigned)p.npix), threads, smem, s, p);
 }
 
 }  // namespace nlos

@@ -38,6 +38,7 @@
 
 #include "nlos_bounds.cuh"
 #include "nlos_internal.h"
+#include "nlos_launch.cuh"
 #include "nlos_umma.cuh"
 
 namespace nlos {
@@ -314,6 +315,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tm = tbase;
+  pdl_wait();
   const WsWork W(p);
   float sa, inv_sa;
   a_scale<Op>(p, sa, inv_sa);
@@ -370,6 +372,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
         if (err) break;
       }
     }
+    pdl_trigger();   // the last operand copies are on their way
   } else if (warp == kMmaWarp) {
     // MMA issue
     if (lane == 0) {
@@ -502,6 +505,8 @@ __global__ void __launch_bounds__(kThreads) pf_umma_kernel(const PfUmmaParams p)
   unsigned char* B = um_sm + S::B_OFF;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int row = tid & (kUmmaTile - 1), half = tid >> 7;
+  pdl_trigger();
+  pdl_wait();
   const int tile = blockIdx.x;
   const int2 i01 = p.tile_i01[tile];
   int pix = p.tile_pix[(size_t)tile * kUmmaTile + row];
@@ -654,8 +659,7 @@ cudaError_t launch_simple(const PfUmmaParams& p, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  k<<<(unsigned)p.ntiles, kThreads, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_kernel(p.after, k, dim3((unsigned)p.ntiles), kThreads, smem, s, p);
 }
 
 int sm_count() {
@@ -704,8 +708,7 @@ cudaError_t launch_ws(const PfUmmaParams& p, cudaStream_t s) {
   const WsShape w = ws_shape(p);
   PfUmmaParams q = p;
   q.split = w.split;
-  k<<<w.grid, kWsThreads, smem, s>>>(q);
-  return cudaGetLastError();
+  return launch_kernel(p.after, k, dim3((unsigned)w.grid), kWsThreads, smem, s, q);
 }
 
 template <class Op>
