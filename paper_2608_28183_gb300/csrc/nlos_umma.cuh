@@ -94,6 +94,15 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
+// 16 lanes (rows) x 16 columns of 32-bit values from tensor memory: thread t of
+// the warp gets columns 2 (t % 4) + {0, 1} (+ 8 for v[4..7]) of row t / 4 in
+// v[0..1] and of row t / 4 + 8 in v[2..3], so that four threads hold eight
+// consecutive columns of a row
+__device__ __forceinline__ void tmem_ld_16x256b_x2(uint32_t addr, uint32_t (&v)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+               : "r"(addr));
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // 1D bulk copy global -> shared completing `bytes` of transaction count on

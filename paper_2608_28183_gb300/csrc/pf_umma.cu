@@ -45,8 +45,9 @@ namespace nlos {
 
 namespace {
 
-constexpr int kWaitLimit = 1 << 26;                    // probes of a barrier (a few hundred ms)
+constexpr int kWaitLimit = 1 << 20;                    // waits on a barrier, each suspended for a while (~1 s in all)
 constexpr uint32_t kSmemBudget = 200 * 1024;           // dynamic shared memory of the stages
+constexpr int kMaxStages = 4;
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -76,14 +77,17 @@ struct OpF16 {
   __device__ static __forceinline__ float2 load(In v) { return __half22float2(v); }
   __device__ static __forceinline__ In zero() { return __floats2half2_rn(0.f, 0.f); }
   // A operand parts of one weight at byte offset off
-  __device__ static __forceinline__ void put(unsigned char* a, uint32_t off, float x, float y) {
-    *reinterpret_cast<__half2*>(a + off) = __floats2half2_rn(x, y);
+  __device__ static __forceinline__ void put(unsigned char* a, uint32_t off, float2 x) {
+    *reinterpret_cast<__half2*>(a + off) = __floats2half2_rn(x.x, x.y);
   }
   __device__ static __forceinline__ uint32_t idesc(int N) { return umma_idesc_f16<false>(kUmmaTile, N); }
   __device__ static __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
     umma_f16(d, a, b, id, acc);
   }
   __device__ static __forceinline__ Out out(float x, float y) { return __floats2half2_rn(x, y); }
+  __device__ static __forceinline__ void store2(Out* p, Out a, Out b) {
+    *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
+  }
 };
 
 struct OpF16x3 {
@@ -98,18 +102,22 @@ struct OpF16x3 {
   static constexpr int kQ = kRowBytes / (2 * kElem);
   __device__ static __forceinline__ float2 load(In v) { return v; }
   __device__ static __forceinline__ In zero() { return make_float2(0.f, 0.f); }
-  // x, y already scaled into f16 range: hi = f16(x), lo = f16(x - hi)
-  __device__ static __forceinline__ void put(unsigned char* a, uint32_t off, float x, float y) {
-    const __half2 hi = __floats2half2_rn(x, y);
+  // x already scaled into f16 range: hi = f16(x), lo = f16(x - hi)
+  __device__ static __forceinline__ void put(unsigned char* a, uint32_t off, float2 x) {
+    const __half2 hi = __floats2half2_rn(x.x, x.y);
     const float2 h = __half22float2(hi);
+    const float2 lo = __fadd2_rn(x, make_float2(-h.x, -h.y));
     *reinterpret_cast<__half2*>(a + off) = hi;
-    *reinterpret_cast<__half2*>(a + kABytes + off) = __floats2half2_rn(x - h.x, y - h.y);
+    *reinterpret_cast<__half2*>(a + kABytes + off) = __floats2half2_rn(lo.x, lo.y);
   }
   __device__ static __forceinline__ uint32_t idesc(int N) { return umma_idesc_f16<false>(kUmmaTile, N); }
   __device__ static __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
     umma_f16(d, a, b, id, acc);
   }
   __device__ static __forceinline__ Out out(float x, float y) { return make_float2(x, y); }
+  __device__ static __forceinline__ void store2(Out* p, Out a, Out b) {
+    *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
+  }
 };
 
 // Scale of the A operand of a scaled kind: 2^(15 - e(amax) - abound_exp)
@@ -146,7 +154,7 @@ struct Sizes {
   static constexpr uint32_t B_BLOCK = Op::kParts * B_BYTES;                    // all parts of one bin
   static constexpr uint32_t B_OFF = 2 * Op::kParts * Op::kABytes;
   static constexpr uint32_t STAGE = B_OFF + 2 * B_BLOCK;
-  static constexpr int STAGES = kSmemBudget / STAGE >= 4 ? 4 : (int)(kSmemBudget / STAGE);
+  static constexpr int STAGES = kSmemBudget / STAGE >= kMaxStages ? kMaxStages : (int)(kSmemBudget / STAGE);
   static constexpr uint32_t ACC_COLS = N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : 256;
   static_assert(STAGES >= 1, "a stage must fit in shared memory");
 };
@@ -165,12 +173,14 @@ struct AChunk {
     r = (T / (Op::kQ / 4)) * 8 + (t & 7);
     q = (T % (Op::kQ / 4)) * 4 + ((t & 31) >> 3);
   }
-  // value v of row r with weights (1 - alpha) sa, alpha sa into both A operands
-  __device__ static __forceinline__ void put(unsigned char* stage, int r, int q, float2 v, float alpha, float sa) {
+  // value v of row r with weights w.x = (1 - alpha) sa, w.y = alpha sa into both A operands
+  __device__ static __forceinline__ void put(unsigned char* stage, int r, int q, float2 v, float2 w) {
     const uint32_t off = chunk_offset<Op>(r, q);
-    const float w0 = (1.f - alpha) * sa, w1 = alpha * sa;
-    Op::put(stage, off, w0 * v.x, w0 * v.y);
-    Op::put(stage + Op::kParts * Op::kABytes, off, w1 * v.x, w1 * v.y);
+    Op::put(stage, off, __fmul2_rn(v, make_float2(w.x, w.x)));
+    Op::put(stage + Op::kParts * Op::kABytes, off, __fmul2_rn(v, make_float2(w.y, w.y)));
+  }
+  __device__ static __forceinline__ float2 weights(float alpha, float sa) {
+    return make_float2((1.f - alpha) * sa, alpha * sa);
   }
 };
 
@@ -197,53 +207,84 @@ __device__ __forceinline__ void mma_chunk(uint32_t acc, uint32_t idesc, const un
   }
 }
 
+// The rows a thread of an epilogue warp stores: row[k] = 8 k + lane / 4 of the
+// warp's 32, with their output rows (nullptr: none) and scales
+template <class Op>
+struct EpiRows {
+  typename Op::Out* crow[4];
+  float gsc[4];
+};
+
 // accumulator rows of one warp -> C (taper and scale), columns [c0, c0 + ncols);
 // `add`: the accumulator holds part of the frequency sum and is added to C
-// (cleared beforehand) with atomics instead of stored
+// (cleared beforehand) with atomics instead of stored. Four threads hold eight
+// consecutive depths of a row, so a store of two complex values per thread
+// covers eight rows in 64-byte (f16: 32-byte) runs; with one row per thread each
+// store touched 32 rows in 16-byte pieces, and the epilogue cost 26 us of
+// 111 at 128x128x1024 float32 (48 of 207 at 256x256x512 f16).
 template <class Op, int Db>
-__device__ __forceinline__ void epilogue_cols(uint32_t acc, int warp, int pix, float gsc, typename Op::Out* crow,
-                                              int blk, int D, int c0, int ncols, bool add = false) {
+__device__ __forceinline__ void epilogue_cols(uint32_t acc, int warp, const EpiRows<Op>& rows, int blk, int D, int c0,
+                                              int ncols, bool add = false) {
   using Out = typename Op::Out;
-  constexpr int kVec = 16 / sizeof(Out);        // complex values per 16-byte store
   const uint32_t lane_base = acc + ((uint32_t)(32 * (warp & 3)) << 16);
+  const int q2 = 2 * (threadIdx.x & 3);
   for (int c = c0; c < c0 + ncols; c += 16) {
-    uint32_t re[16], im[16];
-    tmem_ld16(lane_base + (uint32_t)c, re);
-    tmem_ld16(lane_base + (uint32_t)(Db + c), im);
-    tmem_wait_ld();
-    if (pix >= 0) {
-      Out o[16];
 #pragma unroll
-      for (int q = 0; q < 16; ++q) o[q] = Op::out(gsc * __uint_as_float(re[q]), gsc * __uint_as_float(im[q]));
-      if (add) {
+    for (int half = 0; half < 2; ++half) {      // rows 0-15, 16-31 of the warp's
+      const uint32_t base = lane_base + ((uint32_t)(16 * half) << 16);
+      uint32_t re[8], im[8];
+      tmem_ld_16x256b_x2(base + (uint32_t)c, re);
+      tmem_ld_16x256b_x2(base + (uint32_t)(Db + c), im);
+      tmem_wait_ld();
 #pragma unroll
-        for (int q = 0; q < 16; ++q)
-          if (blk * Db + c + q < D) atomicAdd(crow + c + q, o[q]);
-      } else if (blk * Db + c + 16 <= D && (reinterpret_cast<uintptr_t>(crow + c) & 15) == 0) {
-        uint4* dst = reinterpret_cast<uint4*>(crow + c);
+      for (int g = 0; g < 2; ++g) {             // columns c + 8 g ..
 #pragma unroll
-        for (int v = 0; v < 16 / kVec; ++v) dst[v] = reinterpret_cast<const uint4*>(o)[v];
-      } else {
-#pragma unroll
-        for (int q = 0; q < 16; ++q)
-          if (blk * Db + c + q < D) crow[c + q] = o[q];
+        for (int h = 0; h < 2; ++h) {           // rows t / 4, t / 4 + 8
+          Out* crow = rows.crow[2 * half + h];
+          if (!crow) continue;
+          const float gsc = rows.gsc[2 * half + h];
+          const int k = 4 * g + 2 * h, d = c + 8 * g + q2;
+          const Out o0 = Op::out(gsc * __uint_as_float(re[k]), gsc * __uint_as_float(im[k]));
+          const Out o1 = Op::out(gsc * __uint_as_float(re[k + 1]), gsc * __uint_as_float(im[k + 1]));
+          if (add) {
+            if (blk * Db + d < D) atomicAdd(crow + d, o0);
+            if (blk * Db + d + 1 < D) atomicAdd(crow + d + 1, o1);
+          } else if (blk * Db + d + 2 <= D && (reinterpret_cast<uintptr_t>(crow + d) & (2 * sizeof(Out) - 1)) == 0) {
+            Op::store2(crow + d, o0, o1);
+          } else {
+            if (blk * Db + d < D) crow[d] = o0;
+            if (blk * Db + d + 1 < D) crow[d + 1] = o1;
+          }
+        }
       }
     }
+  }
+}
+
+// rows of `tile` for this thread; g scales every row besides its taper
+template <class Op>
+__device__ __forceinline__ void epilogue_rows(const PfUmmaParams& p, int tile, int blk, int warp, float g, EpiRows<Op>& rows) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const size_t i = (size_t)tile * kUmmaTile + 32 * (warp & 3) + 8 * k + ((threadIdx.x & 31) >> 2);
+    const int pix = p.tile_pix[i];
+    const bool ok = pix >= 0 && bchk((long long)pix * p.D + p.D - 1, p.C_n, p.err);   // the row must lie in C
+    rows.crow[k] = ok ? static_cast<typename Op::Out*>(p.C) + (size_t)pix * p.D + (size_t)blk * p.Db : nullptr;
+    rows.gsc[k] = g * p.tile_acut[i];
   }
 }
 
 // ---------------------------------------------------------------------------
 // Warp-specialised persistent schedule
 // ---------------------------------------------------------------------------
-constexpr int kMaxStages = 4;
 // parts of a tail unit's frequency sum: with at most two, every element of C
 // receives at most two atomic additions onto an exact zero (0 + x is exact,
 // x + y = y + x), so the result does not depend on their order
 constexpr int kMaxSplit = 2;
-constexpr int kWsBuilders = 256;                 // warps 0-7: A build
-constexpr int kProducerWarp = kWsBuilders / 32;  // warp 8: B copies
-constexpr int kMmaWarp = kProducerWarp + 1;      // warp 9: MMA issue
-constexpr int kEpiWarp0 = kMmaWarp + 1;          // warps 10-13: epilogue, one per TMEM lane quarter
+constexpr int kWsBuilders = 512;                 // warps 0-15: A build
+constexpr int kProducerWarp = kWsBuilders / 32;  // warp 16: B copies
+constexpr int kMmaWarp = kProducerWarp + 1;      // warp 17: MMA issue
+constexpr int kEpiWarp0 = kMmaWarp + 1;          // warps 18-21: epilogue, one per TMEM lane quarter
 constexpr int kEpiThreads = 128;
 constexpr int kWsThreads = kWsBuilders + 64 + kEpiThreads;
 
@@ -291,7 +332,6 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
   using S = Sizes<Op, Db>;
   using A = AChunk<Op, kWsBuilders>;
   using In = typename Op::In;
-  using Out = typename Op::Out;
   constexpr int kStages = S::STAGES;
   extern __shared__ __align__(128) unsigned char ws_sm[];
   __shared__ uint64_t full_b[kMaxStages], full_a[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2];
@@ -302,7 +342,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&full_b[s], 1);
-      mbar_init(&full_a[s], kWsBuilders);
+      mbar_init(&full_a[s], kWsBuilders / 32);
       mbar_init(&empty[s], 1);
     }
     for (int a = 0; a < 2; ++a) {
@@ -355,7 +395,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
       for (int kc = sg.k0; kc < sg.k1; ++kc, ++g) {
         const int s = g % kStages, r = g / kStages;
         if (lane == 0) {
-          if (r >= 1 && !mbar_spin_bounded(&empty[s], (r - 1) & 1, kWaitLimit)) err = 1;
+          if (r >= 1 && !mbar_wait_bounded(&empty[s], (r - 1) & 1, kWaitLimit)) err = 1;
           if (!err) {
             unsigned char* b = stage(s) + S::B_OFF;
             mbar_arrive_expect_tx(&full_b[s], 2 * S::B_BLOCK);
@@ -383,9 +423,9 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
         const int a = j & 1;
         for (int kc = sg.k0; kc < sg.k1; ++kc, ++g) {
           const int s = g % kStages, r = g / kStages;
-          if (kc == sg.k0 && j >= 2 && !mbar_spin_bounded(&acc_empty[a], ((j - 2) >> 1) & 1, kWaitLimit)) err = 1;
-          if (!err && !mbar_spin_bounded(&full_b[s], r & 1, kWaitLimit)) err = 1;
-          if (!err && !mbar_spin_bounded(&full_a[s], r & 1, kWaitLimit)) err = 1;
+          if (kc == sg.k0 && j >= 2 && !mbar_wait_bounded(&acc_empty[a], ((j - 2) >> 1) & 1, kWaitLimit)) err = 1;
+          if (!err && !mbar_wait_bounded(&full_b[s], r & 1, kWaitLimit)) err = 1;
+          if (!err && !mbar_wait_bounded(&full_a[s], r & 1, kWaitLimit)) err = 1;
           if (err) break;
           tc_fence_after_sync();
           mma_chunk<Op, Db>(tm + (uint32_t)(a * S::ACC_COLS), idesc, stage(s), kc == sg.k0);
@@ -395,41 +435,39 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
       }
     }
   } else if (warp >= kEpiWarp0) {
-    // epilogue: warp w reads TMEM lane quarter w % 4 (thread = tile row) and
-    // writes every depth of its row; runs beside the next segment's MMAs
-    const int row = 32 * (warp & 3) + lane;
+    // epilogue: warp w reads TMEM lane quarter w % 4 and writes every depth of
+    // its 32 rows; runs beside the next segment's MMAs
     for (int j = 0; j < nseg; ++j) {
       const Seg sg = W.seg(p, j);
       const int a = j & 1;
-      if (!mbar_spin_bounded(&acc_full[a], (j >> 1) & 1, kWaitLimit)) {
+      EpiRows<Op> rows;
+      epilogue_rows<Op>(p, sg.tile, sg.blk, warp, p.scale * inv_sa, rows);
+      if (!mbar_wait_bounded(&acc_full[a], (j >> 1) & 1, kWaitLimit)) {
         err = 1;
         break;
       }
       tc_fence_after_sync();
-      int pix = p.tile_pix[(size_t)sg.tile * kUmmaTile + row];
-      if (pix >= 0 && !bchk((long long)pix * p.D + p.D - 1, p.C_n, p.err)) pix = -1;   // the row must lie in C
-      const float ac = p.tile_acut[(size_t)sg.tile * kUmmaTile + row];
-      Out* crow = static_cast<Out*>(p.C) + (size_t)(pix >= 0 ? pix : 0) * p.D + (size_t)sg.blk * Db;
-      epilogue_cols<Op, Db>(tm + (uint32_t)(a * S::ACC_COLS), warp, pix, p.scale * inv_sa * ac, crow, sg.blk, p.D, 0, Db,
-                            sg.partial);
+      epilogue_cols<Op, Db>(tm + (uint32_t)(a * S::ACC_COLS), warp, rows, sg.blk, p.D, 0, Db, sg.partial);
       tc_fence_before_sync();
       mbar_arrive(&acc_empty[a]);
     }
   } else {
-    // builders: A stages. A builder touches kIters rows: their pixel and
-    // weight are held in registers per segment, and the next chunk's phasors
-    // are loaded before the current chunk is stored
+    // builders: A stages. A builder touches kIters rows of a chunk and keeps
+    // the phasors of the next kAhead chunks in flight in registers, across
+    // segments: with one chunk ahead a step of the pipeline took as long as
+    // the loads' latency plus the build (1.5 us a step in f16)
+    constexpr int kAhead = 2;
     const int t = tid;
     const In* Ph = static_cast<const In*>(p.Phat);
-    int rp[A::kIters];
-    float ra[A::kIters];
+    int rp[A::kIters];            // rows of the load cursor's segment: pixel and weight
+    float2 ra[A::kIters];
     auto load_rows = [&](int tl) {
 #pragma unroll
       for (int i = 0; i < A::kIters; ++i) {
         int r, q;
         A::coords(i, t, r, q);
         rp[i] = p.tile_pix[(size_t)tl * kUmmaTile + r];
-        ra[i] = p.tile_alpha[(size_t)tl * kUmmaTile + r];
+        ra[i] = A::weights(p.tile_alpha[(size_t)tl * kUmmaTile + r], sa);
       }
     };
     auto load_h = [&](In (&h)[A::kIters], int kc) {
@@ -442,18 +480,38 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
                    ? Ph[(size_t)rp[i] * p.F + f] : Op::zero();
       }
     };
-    In hc[A::kIters], hn[A::kIters];
-    if (nseg > 0) {
-      const Seg s0 = W.seg(p, 0);
-      load_rows(s0.tile);
-      load_h(hc, s0.k0);
-    }
-    int g = 0;
-    for (int j = 0; j < nseg && !err; ++j) {
+    int lj = 0, lk = 0;           // load cursor: segment, chunk
+    Seg ls{};
+    auto load_next = [&](In (&h)[A::kIters], float2 (&al)[A::kIters]) {
+      if (lj >= nseg) return;
+      if (lk == 0) {
+        ls = W.seg(p, lj);
+        load_rows(ls.tile);
+      }
+      load_h(h, ls.k0 + lk);
+#pragma unroll
+      for (int i = 0; i < A::kIters; ++i) al[i] = ra[i];
+      if (ls.k0 + ++lk >= ls.k1) {
+        lk = 0;
+        ++lj;
+      }
+    };
+    int total = 0;
+    for (int j = 0; j < nseg; ++j) {
       const Seg sg = W.seg(p, j);
-      for (int kc = sg.k0; kc < sg.k1; ++kc, ++g) {
+      total += sg.k1 - sg.k0;
+    }
+    In h[kAhead][A::kIters];
+    float2 al[kAhead][A::kIters];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) load_next(h[u], al[u]);
+    for (int g0 = 0; g0 < total && !err; g0 += kAhead) {
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u) {
+        const int g = g0 + u;
+        if (g >= total) break;
         const int s = g % kStages, r = g / kStages;
-        if (r >= 1 && !mbar_spin_bounded(&empty[s], (r - 1) & 1, kWaitLimit)) {
+        if (r >= 1 && !mbar_wait_bounded(&empty[s], (r - 1) & 1, kWaitLimit)) {
           err = 1;
           break;
         }
@@ -461,20 +519,12 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
         for (int i = 0; i < A::kIters; ++i) {
           int rr, q;
           A::coords(i, t, rr, q);
-          A::put(stage(s), rr, q, Op::load(hc[i]), ra[i], sa);
+          A::put(stage(s), rr, q, Op::load(h[u][i]), al[u][i]);
         }
         fence_proxy_async_smem();
-        mbar_arrive(&full_a[s]);
-        // next chunk (of this segment or the next one) in flight
-        if (kc + 1 < sg.k1) {
-          load_h(hn, kc + 1);
-        } else if (j + 1 < nseg) {
-          const Seg nx = W.seg(p, j + 1);
-          load_rows(nx.tile);
-          load_h(hn, nx.k0);
-        }
-#pragma unroll
-        for (int i = 0; i < A::kIters; ++i) hc[i] = hn[i];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&full_a[s]);
+        load_next(h[u], al[u]);
       }
     }
   }
@@ -496,7 +546,6 @@ __global__ void __launch_bounds__(kThreads) pf_umma_kernel(const PfUmmaParams p)
   using S = Sizes<Op, Db>;
   using A = AChunk<Op, kThreads>;
   using In = typename Op::In;
-  using Out = typename Op::Out;
   extern __shared__ __align__(128) unsigned char um_sm[];
   __shared__ uint64_t bar_load, bar_mma;
   __shared__ uint32_t tbase;
@@ -504,14 +553,11 @@ __global__ void __launch_bounds__(kThreads) pf_umma_kernel(const PfUmmaParams p)
   __shared__ float salpha[kUmmaTile];
   unsigned char* B = um_sm + S::B_OFF;
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int row = tid & (kUmmaTile - 1), half = tid >> 7;
+  const int half = tid >> 7;
   pdl_trigger();
   pdl_wait();
   const int tile = blockIdx.x;
   const int2 i01 = p.tile_i01[tile];
-  int pix = p.tile_pix[(size_t)tile * kUmmaTile + row];
-  if (pix >= 0 && !bchk((long long)pix * p.D + p.D - 1, p.C_n, p.err)) pix = -1;   // the row must lie in C
-  const float ac = p.tile_acut[(size_t)tile * kUmmaTile + row];
   if (tid < kUmmaTile) {
     spix[tid] = p.tile_pix[(size_t)tile * kUmmaTile + tid];
     salpha[tid] = p.tile_alpha[(size_t)tile * kUmmaTile + tid];
@@ -561,20 +607,20 @@ __global__ void __launch_bounds__(kThreads) pf_umma_kernel(const PfUmmaParams p)
       for (int i = 0; i < A::kIters; ++i) {
         int r, q;
         A::coords(i, tid, r, q);
-        A::put(um_sm, r, q, Op::load(hcur[i]), salpha[r], sa);
+        A::put(um_sm, r, q, Op::load(hcur[i]), A::weights(salpha[r], sa));
       }
       // the next chunk's phasors are in flight while this chunk's MMAs run
       load_h(hnext, kc + 1 < p.KC ? kc + 1 : 0);
       fence_proxy_async_smem();
       __syncthreads();
       if (tid == 0) {
-        ok = mbar_spin_bounded(&bar_load, phase, kWaitLimit);
+        ok = mbar_wait_bounded(&bar_load, phase, kWaitLimit);
         tc_fence_after_sync();
         if (ok) mma_chunk<Op, Db>(dt, idesc, um_sm, kc == 0);
         umma_commit(&bar_mma);
       }
       // the MMAs read A and B; they finish before the next chunk overwrites them
-      const bool done = mbar_spin_bounded(&bar_mma, phase, kWaitLimit);
+      const bool done = mbar_wait_bounded(&bar_mma, phase, kWaitLimit);
       ok = __syncthreads_and(ok && done ? 1 : 0) != 0;
       phase ^= 1;
 #pragma unroll
@@ -584,9 +630,10 @@ __global__ void __launch_bounds__(kThreads) pf_umma_kernel(const PfUmmaParams p)
     if (!ok) break;
     // epilogue: warps w and w + 4 share the rows of lane quarter w % 4
     tc_fence_after_sync();
-    Out* crow = static_cast<Out*>(p.C) + (size_t)(pix >= 0 ? pix : 0) * p.D + (size_t)blk * Db;
-    if (Db >= 32) epilogue_cols<Op, Db>(dt, warp, pix, p.scale * inv_sa * ac, crow, blk, p.D, half * (Db / 2), Db / 2);
-    else if (half == 0) epilogue_cols<Op, Db>(dt, warp, pix, p.scale * inv_sa * ac, crow, blk, p.D, 0, Db);
+    EpiRows<Op> rows;
+    epilogue_rows<Op>(p, tile, blk, warp, p.scale * inv_sa, rows);
+    if (Db >= 32) epilogue_cols<Op, Db>(dt, warp, rows, blk, p.D, half * (Db / 2), Db / 2);
+    else if (half == 0) epilogue_cols<Op, Db>(dt, warp, rows, blk, p.D, 0, Db);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -594,8 +641,8 @@ __global__ void __launch_bounds__(kThreads) pf_umma_kernel(const PfUmmaParams p)
   if (!ok && tid == 0) {
     if (p.err) atomicExch(p.err, kDevErrTmaTimeout);
     // a bounded last chance for copies still in flight into this CTA's buffers
-    mbar_spin_bounded(&bar_load, phase ^ 1, kWaitLimit);
-    mbar_spin_bounded(&bar_mma, phase ^ 1, kWaitLimit);
+    mbar_wait_bounded(&bar_load, phase ^ 1, kWaitLimit);
+    mbar_wait_bounded(&bar_mma, phase ^ 1, kWaitLimit);
   }
   tc_fence_before_sync();
   __syncthreads();
