@@ -179,6 +179,7 @@ struct nlos_plan_s {
   float2* ax = nullptr;
   float2* ay = nullptr;
   // phasor-field tables
+  int Fp = 0;                           // stride of the internal phasor rows (>= F)
   int F = 0, D = 0, k_lo = 0, nchunks = 0, kr_storage = kF32;
   float* w = nullptr;
   float2* phase = nullptr;              // [n] exp(-2 pi i m / n) for photon binning
@@ -639,11 +640,25 @@ nlos_status_t pf_finish(nlos_plan_s* p, const std::vector<float>& w) {
   if ((st = ensure_twiddles(p, Nu)) != NLOS_OK) return st;
   if ((st = ensure_twiddles(p, Nv)) != NLOS_OK) return st;
   const size_t cb = complex_bytes(p->storage);
-  const long long a = p->a, b = p->b, F = p->F, D = p->D;
+  const long long a = p->a, b = p->b, D = p->D;
   const long long U = Nu, V = Nv;
-  const size_t b0 = std::max(a * b * F, U * b * D) * cb;           // P, then the y-inverse output
-  const size_t b1 = std::max(a * V * F, U * V * D) * cb;           // y-transformed P, then C
-  const size_t b2 = U * V * F * cb;                                // Phat
+  auto sizes = [&](long long F, size_t (&s)[3]) {
+    s[0] = std::max(a * b * F, U * b * D) * cb;                    // P, then the y-inverse output
+    s[1] = std::max(a * V * F, U * V * D) * cb;                    // y-transformed P, then C
+    s[2] = U * V * F * cb;                                         // Phat
+    return s[0] + s[1] + s[2];
+  };
+  // phasor rows are padded to a multiple of four values: whole 16-byte loads
+  // in the depth sum and aligned rows for the TMA-staged transforms (the
+  // padding columns are transformed along but never read). Small plans keep
+  // the plain stride where the padding would take their buffers past 32 MiB
+  // (plans that fit nlos_reconstruct_noalloc's fixed scratch keep fitting).
+  size_t plain[3], padded[3];
+  p->Fp = (p->F + 3) & ~3;
+  constexpr size_t kSmall = (size_t(32) << 20) - (size_t(64) << 10);
+  if (sizes(p->F, plain) <= (size_t(32) << 20) && sizes(p->Fp, padded) > kSmall) p->Fp = p->F;
+  sizes(p->Fp, padded);
+  const size_t b0 = padded[0], b1 = padded[1], b2 = padded[2];
   p->off[0] = 0;
   p->off[1] = align256(b0);
   p->off[2] = p->off[1] + align256(b1);
@@ -1052,7 +1067,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
 nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol, char* ws, cudaStream_t s,
                      const void* G0, cudaEvent_t g_read = nullptr) {
   const int st = p->storage;
-  const long long a = p->a, b = p->b, n = p->n, F = p->F, D = p->D;
+  const long long a = p->a, b = p->b, n = p->n, F = p->F, D = p->D, Fp = p->Fp;
   void* b0 = ws + p->off[0];
   void* b1 = ws + p->off[1];
   void* b2 = ws + p->off[2];
@@ -1086,6 +1101,7 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
   bp.L = (int)Lt;
   bp.k_lo = p->k_lo;
   bp.F = (int)F;
+  bp.ldp = (int)Fp;
   bp.npencils = a * b;
   bp.ld_scale = 1.0f;
   bp.ld_dev_scale = s_in;
@@ -1115,6 +1131,7 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
     sp.L = (int)Lt;
     sp.k_lo = p->k_lo;
     sp.F = (int)F;
+    sp.ldp = (int)Fp;
     sp.Lx = (int)Nu;
     sp.Ly = (int)Nv;
     sp.amax = bp.amax;
@@ -1130,14 +1147,17 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
   if (!P_in) NLOS_CU(launch_pf_band(bp, st, s), "pf band transform");
   NLOS_MARK(p, s, sid++);
   // PF2: top-left padding and 2D forward transform (y then x) of every band slice
-  l = axis(st, (int)Nv, a, P, b1, F, b * F, F, Nv * F, F, (int)b, (int)Nv, 0, g2b, p->tw[(int)Nv], p->tiles[sid]);
+  // (caller's phasors have rows of F values)
+  const long long Fi = P_in ? F : Fp;
+  l = axis(st, (int)Nv, a, P, b1, Fi, b * Fi, Fi, Nv * Fp, Fp, (int)b, (int)Nv, 0, g2b, p->tw[(int)Nv], p->tiles[sid]);
   l.err = err;
   attach_tmap(l);
   set_extents(l, P_in ? a * b * F : ws_extent(p, 0), ws_extent(p, 1));
   l.after = !P_in;
   NLOS_CU(launch_axis_fft(l, s), "pf y-forward");
   NLOS_MARK(p, s, sid++);
-  l = axis(st, (int)Nu, 1, b1, b2, Nv * F, 0, Nv * F, 0, Nv * F, (int)a, (int)Nu, 0, g2a, p->tw[(int)Nu], p->tiles[sid]);
+  l = axis(st, (int)Nu, 1, b1, b2, Nv * Fp, 0, Nv * Fp, 0, Nv * Fp, (int)a, (int)Nu, 0, g2a, p->tw[(int)Nu],
+           p->tiles[sid]);
   l.err = err;
   attach_tmap(l);
   set_extents(l, ws_extent(p, 1), ws_extent(p, 2));
@@ -1147,7 +1167,7 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
   }
   if (p->d.method == NLOS_PHASOR_DENSE) {
     // PF3, dense kernel: C = sum_f Phat * Khat (Alg. 3), every pixel written
-    PfDenseParams dp{!g_read, static_cast<const float2*>(b2), p->Kd, static_cast<float2*>(b1), Nu * Nv, (int)F, (int)D};
+    PfDenseParams dp{!g_read, static_cast<const float2*>(b2), p->Kd, static_cast<float2*>(b1), Nu * Nv, (int)F, (int)D, (int)Fp};
     NLOS_CU(launch_pf_dense(dp, s), "pf dense depth sum");
   } else {
     // PF3: depth sum (pixels beyond the cutoff stay zero); f16 and float32
@@ -1169,6 +1189,7 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
       up.tile_acut = p->tu_acut;
       up.ntiles = p->ntiles_u;
       up.F = (int)F;
+      up.ldp = (int)Fp;
       up.D = (int)D;
       up.Db = p->Db_u;
       up.nblk = p->nblk_u;
@@ -1214,6 +1235,7 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
     dp.chunk_acut = p->ch_acut;
     dp.nchunks = p->nchunks;
     dp.F = (int)F;
+    dp.ldp = (int)Fp;
     dp.D = (int)D;
     dp.scale = c3;
     NLOS_CU(launch_pf_depth(dp, st, p->kr_storage, s), "pf depth sum");
@@ -1569,6 +1591,7 @@ nlos_status_t nlos_bin_phasors(nlos_plan_t p, const uint32_t* pixel, const uint3
     bp.L = p->Lt;
     bp.k_lo = p->k_lo;
     bp.F = p->F;
+    bp.ldp = p->F;
     bp.npencils = (long long)p->a * p->b;
     bp.ld_scale = 1.0f;
     bp.st_scale = 1.0f;

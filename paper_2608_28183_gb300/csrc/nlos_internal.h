@@ -203,6 +203,7 @@ struct PfBandParams {
   const float2* tw;            // twiddles for L
   const float* w;              // [F]
   int n, k_lo, F;              // n: samples per pencil (stride of H)
+  int ldp;                     // stride of P's pencils (>= F)
   int L;                       // DFT length (power of two >= n; samples beyond n are zero)
   long long npencils;          // a * b
   float ld_scale;
@@ -224,10 +225,10 @@ cudaError_t launch_pf_band(const PfBandParams& p, int storage, cudaStream_t s);
 // Phat(Lx - kx, -ky, f) = w(f) conj(Z(L - k_lo - f)). Float32 only.
 struct PfSpecParams {
   const float2* G;             // [Lx/2 + 1][Ly][n]
-  float2* Phat;                // [Lx][Ly][F]
+  float2* Phat;                // [Lx][Ly][ldp], ldp >= F
   const float2* tw;            // twiddles for L
   const float* w;              // [F]
-  int n, L, k_lo, F, Lx, Ly;
+  int n, L, k_lo, F, ldp, Lx, Ly;
   unsigned* amax;              // when set: atomicMax of max |Re|, |Im| of the stored Phat (float bits)
   long long G_n, Phat_n;       // element extents (bounds-checked build; 0: unchecked)
   int* err;                    // device error word (bounds-checked build), may be null
@@ -259,14 +260,14 @@ cudaError_t launch_bin_transient(const uint32_t* pixel, const uint32_t* ticks, l
 constexpr int kPfChunk = 16;
 struct PfDepthParams {
   bool after;                  // launched after another kernel of the same call (nlos_launch.cuh)
-  const void* Phat;            // [Nu*Nv][F] complex (storage type)
+  const void* Phat;            // [Nu*Nv][ldp] complex (storage type), ldp >= F
   const void* K;               // [N_rho][F][D] complex (kernel storage type)
   void* C;                     // [Nu*Nv][D] complex (storage type)
   const int2* chunk_i01;       // [nchunks] (i0, i1)
   const int* chunk_pix;        // [nchunks][16] pixel index or -1
   const float* chunk_alpha;    // [nchunks][16]
   const float* chunk_acut;     // [nchunks][16]
-  int nchunks, F, D;
+  int nchunks, F, D, ldp;
   float scale;
   const float* dev_scale;      // optional device scalar multiplying C
 };
@@ -310,7 +311,7 @@ __host__ __device__ constexpr int umma_chunk_cols(int) { return 32; }
 __host__ __device__ constexpr int umma_parts(int kind) { return kind == kUmmaF16 ? 1 : 2; }
 struct PfUmmaParams {
   bool after;                  // launched after another kernel of the same call (nlos_launch.cuh)
-  const void* Phat;            // [npix][F] half2 (f16 kind) or float2 (f16x3 kind)
+  const void* Phat;            // [npix][ldp] half2 (f16 kind) or float2 (f16x3 kind), ldp >= F
   const void* B;               // [n_rho][nblk][KC][parts][2 Db rows x row bytes], operand layout
   void* C;                     // [npix][D] half2 or float2
   const int2* tile_i01;        // [ntiles]
@@ -318,6 +319,7 @@ struct PfUmmaParams {
   const float* tile_alpha;     // [ntiles][128]
   const float* tile_acut;      // [ntiles][128]
   int ntiles, F, D, Db, nblk, KC;
+  int ldp;                     // a multiple of 4 (the operand builders load 16 bytes at a time) or F
   int kind;                    // UmmaKind
   int split;                   // set by the launcher: parts of a tail unit's frequency sum
   // kUmmaF16x3 only: *amax (float bits) bounds |Re|, |Im| of the compact
@@ -361,11 +363,11 @@ cudaError_t launch_dense_gen(const DenseGenParams& p, cudaStream_t s);
 // Dense depth sum: C[pix][d] = sum_f Phat[pix][f] * Khat[pix][f][d] (float32).
 struct PfDenseParams {
   bool after;                  // launched after another kernel of the same call (nlos_launch.cuh)
-  const float2* Phat;          // [npix][F]
+  const float2* Phat;          // [npix][ldp], ldp >= F
   const float2* K;             // [npix][F][D]
   float2* C;                   // [npix][D]
   long long npix;
-  int F, D;
+  int F, D, ldp;
 };
 cudaError_t launch_pf_dense(const PfDenseParams& p, cudaStream_t s);
 

@@ -75,19 +75,19 @@ template <class TS>
 __device__ __forceinline__ float band_split_store(const PfBandParams& p, const float2* O, long long q, bool has1,
                                                   int j0, int TPC) {
   float m = 0.f;
-  TS* P0 = static_cast<TS*>(p.P) + q * p.F;
-  TS* P1 = P0 + p.F;
+  TS* P0 = static_cast<TS*>(p.P) + q * p.ldp;
+  TS* P1 = P0 + p.ldp;
   for (int f = j0; f < p.F; f += TPC) {
     const float2 z = O[f], c = cconj(O[p.F + f]);
     const float s = 0.5f * __ldg(p.w + f) * p.st_scale;
     float2 x0 = make_float2(s * (z.x + c.x), s * (z.y + c.y));
     float2 x1 = make_float2(s * (z.y - c.y), -s * (z.x - c.x));   // (z - c) / (2i)
-    if (bchk(q * p.F + f, p.P_n, p.err)) {
+    if (bchk(q * p.ldp + f, p.P_n, p.err)) {
       if (p.accumulate) x0 = cadd(x0, Cpx<TS>::get(P0 + f));
       Cpx<TS>::put(P0 + f, x0);
       m = fmaxf(m, fmaxf(fabsf(x0.x), fabsf(x0.y)));
     }
-    if (has1 && bchk((q + 1) * p.F + f, p.P_n, p.err)) {
+    if (has1 && bchk((q + 1) * p.ldp + f, p.P_n, p.err)) {
       if (p.accumulate) x1 = cadd(x1, Cpx<TS>::get(P1 + f));
       Cpx<TS>::put(P1 + f, x1);
       m = fmaxf(m, fmaxf(fabsf(x1.x), fabsf(x1.y)));
@@ -262,7 +262,7 @@ static cudaError_t launch_band_typed(const PfBandParams& p, cudaStream_t s) {
 }
 
 cudaError_t launch_pf_band(const PfBandParams& p, int storage, cudaStream_t s) {
-  if (p.npencils <= 0 || p.F <= 0) return cudaErrorInvalidValue;
+  if (p.npencils <= 0 || p.F <= 0 || p.ldp < p.F) return cudaErrorInvalidValue;
   switch (storage) {
     case kF32: return launch_band_typed<float, float2>(p, s);
     case kF16: return launch_band_typed<__half, __half2>(p, s);
@@ -329,8 +329,8 @@ pf_band_spectrum_kernel(const PfSpecParams p) {
   const long long q = valid ? pid : 0;
   const int kx = (int)(q / p.Ly);
   const int ky = (int)(q % p.Ly);
-  const long long o0 = q * p.F;                     // (kx Ly + ky) F
-  const long long o1 = ((long long)(p.Lx - kx) * p.Ly + ((p.Ly - ky) & (p.Ly - 1))) * p.F;
+  const long long o0 = q * p.ldp;                   // (kx Ly + ky) ldp
+  const long long o1 = ((long long)(p.Lx - kx) * p.Ly + ((p.Ly - ky) & (p.Ly - 1))) * p.ldp;
   const bool partner = kx > 0 && 2 * kx < p.Lx;
   PfSpecCtx<L> ctx{p.G + q * p.n, p.Phat + o0, partner ? p.Phat + o1 : nullptr, pfs_sm + w * S::SMEM, p.tw, p.w,
                    p.k_lo, p.F, p.n, valid, q * p.n, p.G_n, o0, o1, p.Phat_n, p.err};
@@ -362,7 +362,7 @@ static cudaError_t launch_spec_one(const PfSpecParams& p, cudaStream_t s) {
 }
 
 cudaError_t launch_pf_band_spectrum(const PfSpecParams& p, cudaStream_t s) {
-  if (p.F <= 0 || p.n <= 0 || p.n > p.L || p.Lx < 2 || p.Ly < 1 || (p.Ly & (p.Ly - 1)) ||
+  if (p.F <= 0 || p.ldp < p.F || p.n <= 0 || p.n > p.L || p.Lx < 2 || p.Ly < 1 || (p.Ly & (p.Ly - 1)) ||
       p.k_lo < 1 || p.k_lo + p.F > p.L / 2)
     return cudaErrorInvalidValue;
   switch (p.L) {
@@ -413,7 +413,7 @@ pf_depth_kernel(const PfDepthParams p) {
   for (int idx = threadIdx.x; idx < kPfChunk * F; idx += kDepthThreads) {
     const int q = idx / F, f = idx - q * F;
     const int px = pix[q];
-    ps[f * kPfChunk + q] = px >= 0 ? Cpx<TS>::get(Ph + (long long)px * F + f) : make_float2(0.f, 0.f);
+    ps[f * kPfChunk + q] = px >= 0 ? Cpx<TS>::get(Ph + (long long)px * p.ldp + f) : make_float2(0.f, 0.f);
   }
   __syncthreads();
   float alpha[kPfChunk];
@@ -487,7 +487,7 @@ static cudaError_t launch_depth_typed(const PfDepthParams& p, cudaStream_t s) {
 
 cudaError_t launch_pf_depth(const PfDepthParams& p, int storage, int kstorage, cudaStream_t s) {
   if (p.nchunks <= 0) return cudaSuccess;
-  if (p.F <= 0 || p.D <= 0 || p.D > 65535 * kDepthBlock) return cudaErrorInvalidValue;
+  if (p.F <= 0 || p.ldp < p.F || p.D <= 0 || p.D > 65535 * kDepthBlock) return cudaErrorInvalidValue;
   if (storage == kF32 && kstorage == kF32) return launch_depth_typed<float2, float2>(p, s);
   if (storage == kF16 && kstorage == kF16) return launch_depth_typed<__half2, __half2>(p, s);
   if (storage == kBF16 && kstorage == kBF16) return launch_depth_typed<__nv_bfloat162, __nv_bfloat162>(p, s);
@@ -786,7 +786,7 @@ __global__ void __launch_bounds__(128) pf_dense_kernel(const PfDenseParams p) {
   pdl_trigger();
   pdl_wait();
   const long long pix = blockIdx.x;
-  for (int f = threadIdx.x; f < p.F; f += blockDim.x) ph_sm[f] = p.Phat[pix * p.F + f];
+  for (int f = threadIdx.x; f < p.F; f += blockDim.x) ph_sm[f] = p.Phat[pix * p.ldp + f];
   __syncthreads();
   const float2* K = p.K + pix * p.F * (long long)p.D;
   for (int d = threadIdx.x; d < p.D; d += blockDim.x) {
@@ -871,7 +871,7 @@ cudaError_t launch_clear_rows(void* C, const int* list, long long n, size_t row_
 }
 
 cudaError_t launch_pf_dense(const PfDenseParams& p, cudaStream_t s) {
-  if (p.npix <= 0 || p.F <= 0 || p.D <= 0) return cudaErrorInvalidValue;
+  if (p.npix <= 0 || p.F <= 0 || p.ldp < p.F || p.D <= 0) return cudaErrorInvalidValue;
   const int threads = p.D <= 64 ? 64 : 128;
   const size_t smem = sizeof(float2) * p.F;
   if (smem > 48 * 1024) {

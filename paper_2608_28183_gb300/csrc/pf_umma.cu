@@ -76,9 +76,12 @@ struct OpF16 {
   static constexpr int kQ = kRowBytes / (2 * kElem);        // frequencies per chunk
   __device__ static __forceinline__ float2 load(In v) { return __half22float2(v); }
   __device__ static __forceinline__ In zero() { return __floats2half2_rn(0.f, 0.f); }
-  // A operand parts of one weight at byte offset off
-  __device__ static __forceinline__ void put(unsigned char* a, uint32_t off, float2 x) {
-    *reinterpret_cast<__half2*>(a + off) = __floats2half2_rn(x.x, x.y);
+  // A operand parts of one weight at byte offset off: four values, 16 bytes a part
+  __device__ static __forceinline__ void put4(unsigned char* a, uint32_t off, const float2 (&x)[4]) {
+    __half2 h[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) h[k] = __floats2half2_rn(x[k].x, x[k].y);
+    *reinterpret_cast<uint4*>(a + off) = *reinterpret_cast<const uint4*>(h);
   }
   __device__ static __forceinline__ uint32_t idesc(int N) { return umma_idesc_f16<false>(kUmmaTile, N); }
   __device__ static __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
@@ -103,12 +106,17 @@ struct OpF16x3 {
   __device__ static __forceinline__ float2 load(In v) { return v; }
   __device__ static __forceinline__ In zero() { return make_float2(0.f, 0.f); }
   // x already scaled into f16 range: hi = f16(x), lo = f16(x - hi)
-  __device__ static __forceinline__ void put(unsigned char* a, uint32_t off, float2 x) {
-    const __half2 hi = __floats2half2_rn(x.x, x.y);
-    const float2 h = __half22float2(hi);
-    const float2 lo = __fadd2_rn(x, make_float2(-h.x, -h.y));
-    *reinterpret_cast<__half2*>(a + off) = hi;
-    *reinterpret_cast<__half2*>(a + kABytes + off) = __floats2half2_rn(lo.x, lo.y);
+  __device__ static __forceinline__ void put4(unsigned char* a, uint32_t off, const float2 (&x)[4]) {
+    __half2 hi[4], lo[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      hi[k] = __floats2half2_rn(x[k].x, x[k].y);
+      const float2 h = __half22float2(hi[k]);
+      const float2 d = __fadd2_rn(x[k], make_float2(-h.x, -h.y));
+      lo[k] = __floats2half2_rn(d.x, d.y);
+    }
+    *reinterpret_cast<uint4*>(a + off) = *reinterpret_cast<const uint4*>(hi);
+    *reinterpret_cast<uint4*>(a + kABytes + off) = *reinterpret_cast<const uint4*>(lo);
   }
   __device__ static __forceinline__ uint32_t idesc(int N) { return umma_idesc_f16<false>(kUmmaTile, N); }
   __device__ static __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
@@ -159,25 +167,52 @@ struct Sizes {
   static_assert(STAGES >= 1, "a stage must fit in shared memory");
 };
 
-// A chunk of a tile: frequency q of row r for thread t and iteration i. A
-// warp instruction covers 8 rows x 4 consecutive q: the 32 lanes hit 32
-// distinct shared-memory banks and read 8 runs of 4 consecutive phasors. NT threads (a multiple of
-// 32) share the chunk.
+// A chunk of a tile in groups of four consecutive frequencies q .. q + 3 of a
+// row r, 16 bytes of an operand part: group i of thread t. A warp covers 8
+// rows x 4 groups, so that eight lanes store one 128-byte core matrix, and its
+// 16-byte loads read whole 64-byte (float32: 128-byte) runs of 8 rows.
+// With one frequency per lane the builders, the busiest part of the pipeline,
+// executed three times as many loads and stores. NT threads (a multiple of 32) share
+// the chunk.
 template <class Op, int NT>
 struct AChunk {
-  static constexpr int kBlocks = (kUmmaTile / 8) * (Op::kQ / 4);
+  using In = typename Op::In;
+  static_assert(Op::kQ == 16, "a chunk is 16 frequencies");
+  static constexpr int kBlocks = kUmmaTile / 8;              // of 8 rows x 4 groups
   static constexpr int kIters = kBlocks / (NT / 32);
   static_assert(kIters * (NT / 32) == kBlocks, "threads must divide the chunk");
-  __device__ static __forceinline__ void coords(int i, int t, int& r, int& q) {
-    const int T = i * (NT / 32) + (t >> 5);
-    r = (T / (Op::kQ / 4)) * 8 + (t & 7);
-    q = (T % (Op::kQ / 4)) * 4 + ((t & 31) >> 3);
+  __device__ static __forceinline__ int row(int i, int t) { return (i * (NT / 32) + (t >> 5)) * 8 + (t & 7); }
+  __device__ static __forceinline__ int freq(int t) { return ((t & 31) >> 3) * 4; }
+  // four phasors of pixel pix (< 0: none) from frequency f on; zero beyond F
+  __device__ static __forceinline__ void load(const PfUmmaParams& p, In (&h)[4], int pix, int f) {
+    const In* src = static_cast<const In*>(p.Phat) + (long long)pix * p.ldp + f;
+    if (pix >= 0 && f + 4 <= p.F && (p.ldp & 3) == 0) {
+      if (bchk((long long)pix * p.ldp + f + 3, p.Phat_n, p.err)) {
+        constexpr int kV = 4 * sizeof(In) / 16;              // 16-byte loads
+        uint4 v[kV];
+#pragma unroll
+        for (int k = 0; k < kV; ++k) v[k] = __ldg(reinterpret_cast<const uint4*>(src) + k);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) h[k] = reinterpret_cast<const In*>(v)[k];
+        return;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      h[k] = (pix >= 0 && f + k < p.F && bchk((long long)pix * p.ldp + f + k, p.Phat_n, p.err)) ? src[k] : Op::zero();
   }
-  // value v of row r with weights w.x = (1 - alpha) sa, w.y = alpha sa into both A operands
-  __device__ static __forceinline__ void put(unsigned char* stage, int r, int q, float2 v, float2 w) {
+  // the group's values with weights w.x = (1 - alpha) sa, w.y = alpha sa into both A operands
+  __device__ static __forceinline__ void put(unsigned char* stage, int r, int q, const In (&h)[4], float2 w) {
     const uint32_t off = chunk_offset<Op>(r, q);
-    Op::put(stage, off, __fmul2_rn(v, make_float2(w.x, w.x)));
-    Op::put(stage + Op::kParts * Op::kABytes, off, __fmul2_rn(v, make_float2(w.y, w.y)));
+    float2 x0[4], x1[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 v = Op::load(h[k]);
+      x0[k] = __fmul2_rn(v, make_float2(w.x, w.x));
+      x1[k] = __fmul2_rn(v, make_float2(w.y, w.y));
+    }
+    Op::put4(stage, off, x0);
+    Op::put4(stage + Op::kParts * Op::kABytes, off, x1);
   }
   __device__ static __forceinline__ float2 weights(float alpha, float sa) {
     return make_float2((1.f - alpha) * sa, alpha * sa);
@@ -367,52 +402,50 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
     // the MMAs and, for the f16x3 kind (two stages of 96 KB), asks L2 for the
     // B blocks kPrefetch chunks ahead
     const size_t blk_bytes = (size_t)p.KC * S::B_BLOCK;
-    const unsigned char* Bg = static_cast<const unsigned char*>(p.B);
-    auto b_block = [&](const Seg& sg, int kc, int bin) {
-      const int2 i01 = p.tile_i01[sg.tile];
-      const int b = bin ? i01.y : i01.x;
-      return Bg + ((size_t)b * p.nblk + sg.blk) * blk_bytes + (size_t)kc * S::B_BLOCK;
-    };
-    // prefetch cursor: kPrefetch chunks ahead of the copies
-    constexpr int kPrefetch = 2 * kStages;
-    int pj = 0, pk = 0;
-    Seg ps{};
-    if (nseg > 0) {
-      ps = W.seg(p, 0);
-      pk = ps.k0;
-    }
-    auto advance = [&]() {
-      if (pj >= nseg) return;
-      if (++pk >= ps.k1 && ++pj < nseg) {
-        ps = W.seg(p, pj);
-        pk = ps.k0;
-      }
-    };
-    for (int i = 0; i < kPrefetch; ++i) advance();
-    int g = 0;
-    for (int j = 0; j < nseg && !err; ++j) {
-      const Seg sg = W.seg(p, j);
-      for (int kc = sg.k0; kc < sg.k1; ++kc, ++g) {
-        const int s = g % kStages, r = g / kStages;
-        if (lane == 0) {
-          if (r >= 1 && !mbar_wait_bounded(&empty[s], (r - 1) & 1, kWaitLimit)) err = 1;
-          if (!err) {
-            unsigned char* b = stage(s) + S::B_OFF;
-            mbar_arrive_expect_tx(&full_b[s], 2 * S::B_BLOCK);
-            bulk_load(b, b_block(sg, kc, 0), S::B_BLOCK, &full_b[s]);
-            bulk_load(b + S::B_BLOCK, b_block(sg, kc, 1), S::B_BLOCK, &full_b[s]);
-            if (Op::kPrefetchB && pj < nseg) {
-              bulk_prefetch_l2(b_block(ps, pk, 0), S::B_BLOCK);
-              bulk_prefetch_l2(b_block(ps, pk, 1), S::B_BLOCK);
-            }
-          }
+    if (lane == 0) {
+      // a cursor over the chunks: the two bins' blocks, looked up once per segment
+      struct Cursor {
+        int j = -1, k = 0, k1 = 0;
+        const unsigned char *b0 = nullptr, *b1 = nullptr;
+      };
+      auto advance = [&](Cursor& c) {   // false: past the last chunk
+        if (c.j >= 0 && ++c.k < c.k1) {
+          c.b0 += S::B_BLOCK;
+          c.b1 += S::B_BLOCK;
+          return true;
         }
-        advance();
-        err = __shfl_sync(0xffffffffu, err, 0);
-        if (err) break;
+        if (c.j >= nseg || ++c.j >= nseg) return false;
+        const Seg sg = W.seg(p, c.j);
+        const int2 i01 = p.tile_i01[sg.tile];
+        const unsigned char* Bg = static_cast<const unsigned char*>(p.B) + sg.blk * blk_bytes + (size_t)sg.k0 * S::B_BLOCK;
+        c.b0 = Bg + (size_t)i01.x * p.nblk * blk_bytes;
+        c.b1 = Bg + (size_t)i01.y * p.nblk * blk_bytes;
+        c.k = sg.k0;
+        c.k1 = sg.k1;
+        return true;
+      };
+      // prefetch cursor: kPrefetch chunks ahead of the copies
+      constexpr int kPrefetch = 2 * kStages;
+      Cursor cur, pre;
+      bool more = Op::kPrefetchB;
+      for (int i = 0; i < kPrefetch && more; ++i) more = advance(pre);
+      for (int g = 0; advance(cur); ++g) {
+        const int s = g % kStages, r = g / kStages;
+        if (r >= 1 && !mbar_wait_bounded(&empty[s], (r - 1) & 1, kWaitLimit)) {
+          err = 1;
+          break;
+        }
+        unsigned char* b = stage(s) + S::B_OFF;
+        mbar_arrive_expect_tx(&full_b[s], 2 * S::B_BLOCK);
+        bulk_load(b, cur.b0, S::B_BLOCK, &full_b[s]);
+        bulk_load(b + S::B_BLOCK, cur.b1, S::B_BLOCK, &full_b[s]);
+        if (more && (more = advance(pre))) {
+          bulk_prefetch_l2(pre.b0, S::B_BLOCK);
+          bulk_prefetch_l2(pre.b1, S::B_BLOCK);
+        }
       }
+      pdl_trigger();   // the last operand copies are on their way
     }
-    pdl_trigger();   // the last operand copies are on their way
   } else if (warp == kMmaWarp) {
     // MMA issue
     if (lane == 0) {
@@ -457,40 +490,30 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
     // segments: with one chunk ahead a step of the pipeline took as long as
     // the loads' latency plus the build (1.5 us a step in f16)
     constexpr int kAhead = 2;
-    const int t = tid;
-    const In* Ph = static_cast<const In*>(p.Phat);
+    const int t = tid, q0 = A::freq(t);
     int rp[A::kIters];            // rows of the load cursor's segment: pixel and weight
     float2 ra[A::kIters];
     auto load_rows = [&](int tl) {
 #pragma unroll
       for (int i = 0; i < A::kIters; ++i) {
-        int r, q;
-        A::coords(i, t, r, q);
-        rp[i] = p.tile_pix[(size_t)tl * kUmmaTile + r];
-        ra[i] = A::weights(p.tile_alpha[(size_t)tl * kUmmaTile + r], sa);
-      }
-    };
-    auto load_h = [&](In (&h)[A::kIters], int kc) {
-#pragma unroll
-      for (int i = 0; i < A::kIters; ++i) {
-        int r, q;
-        A::coords(i, t, r, q);
-        const int f = kc * Op::kQ + q;
-        h[i] = (rp[i] >= 0 && f < p.F && bchk((long long)rp[i] * p.F + f, p.Phat_n, p.err))
-                   ? Ph[(size_t)rp[i] * p.F + f] : Op::zero();
+        const size_t r = (size_t)tl * kUmmaTile + A::row(i, t);
+        rp[i] = p.tile_pix[r];
+        ra[i] = A::weights(p.tile_alpha[r], sa);
       }
     };
     int lj = 0, lk = 0;           // load cursor: segment, chunk
     Seg ls{};
-    auto load_next = [&](In (&h)[A::kIters], float2 (&al)[A::kIters]) {
+    auto load_next = [&](In (&h)[A::kIters][4], float2 (&al)[A::kIters]) {
       if (lj >= nseg) return;
       if (lk == 0) {
         ls = W.seg(p, lj);
         load_rows(ls.tile);
       }
-      load_h(h, ls.k0 + lk);
 #pragma unroll
-      for (int i = 0; i < A::kIters; ++i) al[i] = ra[i];
+      for (int i = 0; i < A::kIters; ++i) {
+        A::load(p, h[i], rp[i], (ls.k0 + lk) * Op::kQ + q0);
+        al[i] = ra[i];
+      }
       if (ls.k0 + ++lk >= ls.k1) {
         lk = 0;
         ++lj;
@@ -501,7 +524,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
       const Seg sg = W.seg(p, j);
       total += sg.k1 - sg.k0;
     }
-    In h[kAhead][A::kIters];
+    In h[kAhead][A::kIters][4];
     float2 al[kAhead][A::kIters];
 #pragma unroll
     for (int u = 0; u < kAhead; ++u) load_next(h[u], al[u]);
@@ -516,11 +539,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
           break;
         }
 #pragma unroll
-        for (int i = 0; i < A::kIters; ++i) {
-          int rr, q;
-          A::coords(i, t, rr, q);
-          A::put(stage(s), rr, q, Op::load(h[u][i]), al[u][i]);
-        }
+        for (int i = 0; i < A::kIters; ++i) A::put(stage(s), A::row(i, t), q0, h[u][i], al[u][i]);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&full_a[s]);
@@ -562,7 +581,6 @@ __global__ void __launch_bounds__(kThreads) pf_umma_kernel(const PfUmmaParams p)
     spix[tid] = p.tile_pix[(size_t)tile * kUmmaTile + tid];
     salpha[tid] = p.tile_alpha[(size_t)tile * kUmmaTile + tid];
   }
-  const In* Ph = static_cast<const In*>(p.Phat);
   if (warp == 0) tmem_alloc(&tbase, S::ACC_COLS);
   if (tid == 0) {
     mbar_init(&bar_load, 1);
@@ -572,18 +590,12 @@ __global__ void __launch_bounds__(kThreads) pf_umma_kernel(const PfUmmaParams p)
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
-  auto load_h = [&](In (&h)[A::kIters], int kc) {
+  const int q0 = A::freq(tid);
+  auto load_h = [&](In (&h)[A::kIters][4], int kc) {
 #pragma unroll
-    for (int i = 0; i < A::kIters; ++i) {
-      int r, q;
-      A::coords(i, tid, r, q);
-      const int f = kc * Op::kQ + q;
-      const int px = spix[r];
-      h[i] = (px >= 0 && f < p.F && bchk((long long)px * p.F + f, p.Phat_n, p.err)) ? Ph[(size_t)px * p.F + f]
-                                                                                      : Op::zero();
-    }
+    for (int i = 0; i < A::kIters; ++i) A::load(p, h[i], spix[A::row(i, tid)], kc * Op::kQ + q0);
   };
-  In hcur[A::kIters], hnext[A::kIters];
+  In hcur[A::kIters][4], hnext[A::kIters][4];
   load_h(hcur, 0);
   float sa, inv_sa;
   a_scale<Op>(p, sa, inv_sa);
@@ -605,9 +617,8 @@ __global__ void __launch_bounds__(kThreads) pf_umma_kernel(const PfUmmaParams p)
       }
 #pragma unroll
       for (int i = 0; i < A::kIters; ++i) {
-        int r, q;
-        A::coords(i, tid, r, q);
-        A::put(um_sm, r, q, Op::load(hcur[i]), A::weights(salpha[r], sa));
+        const int r = A::row(i, tid);
+        A::put(um_sm, r, q0, hcur[i], A::weights(salpha[r], sa));
       }
       // the next chunk's phasors are in flight while this chunk's MMAs run
       load_h(hnext, kc + 1 < p.KC ? kc + 1 : 0);
@@ -624,7 +635,9 @@ __global__ void __launch_bounds__(kThreads) pf_umma_kernel(const PfUmmaParams p)
       ok = __syncthreads_and(ok && done ? 1 : 0) != 0;
       phase ^= 1;
 #pragma unroll
-      for (int i = 0; i < A::kIters; ++i) hcur[i] = hnext[i];
+      for (int i = 0; i < A::kIters; ++i)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) hcur[i][k] = hnext[i][k];
       if (!ok) break;
     }
     if (!ok) break;
