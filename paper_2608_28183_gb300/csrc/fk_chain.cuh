@@ -30,6 +30,8 @@
 // alone took 295 us of 393 at 256x256x512 float32, and 260 of 428 in f16.
 // The writers pay with 64-byte (32-byte) segments, which L2 merges.
 #pragma once
+#include <type_traits>
+
 #include "axis_fft.cuh"
 #include "nlos_bounds.cuh"
 #include "nlos_internal.h"
@@ -38,7 +40,16 @@
 namespace nlos {
 
 constexpr int kChainIC = 8;                // columns per sub-tile
-constexpr int kChainE = 32;                // values per thread (radix-32 passes)
+// values per thread of the L-point transforms. 512 and 1024 points take two
+// radix-32 passes (three of radix 16). 128 and 256 points take two passes
+// either way; with 16 values per thread (about 64 registers against 168) a
+// 256-point CTA has four transforming warps instead of two and six CTAs fit
+// an SM instead of four: at 128x128x512 float32 the inverse pair takes 95.5 us against
+// 100.7, the forward pair 74.5 against 84.8. 16-bit
+// storage keeps 32, and with it its roundings.
+template <int L, class TS> constexpr int chain_e() {
+  return L <= 256 && sizeof(TS) == 8 ? 16 : 32;
+}
 constexpr int kChainCols = 2 * kChainIC;   // columns (t or z values) per chunk and item
 constexpr int kChainWaitLimit = 1 << 18;   // polls of a chunk counter (~0.1 s with the back-off; below the ~1 s slot waits)
 
@@ -81,14 +92,19 @@ struct ChainSlot {
   int ticket, sub;
 };
 
-template <int L, int NSLOT = 2> struct ChainTile {
-  static constexpr int CONSUMERS = kChainIC * (L / kChainE);   // threads that transform
+template <int L, int E, int NSLOT = 2> struct ChainTile {
+  static constexpr int CONSUMERS = kChainIC * (L / E);         // threads that transform
   static constexpr int THREADS = CONSUMERS + 32;               // + the producer warp
-  static constexpr size_t BUF = sizeof(float2) * FftShape<L, kChainE>::SMEM * kChainIC;   // multiple of 128 bytes
-  static constexpr size_t TW = sizeof(float2) * FftShape<L, kChainE>::TWSIZE;   // the twiddle table's copy
+  static constexpr size_t BUF = sizeof(float2) * FftShape<L, E>::SMEM * kChainIC;   // multiple of 128 bytes
+  static constexpr size_t TW = sizeof(float2) * FftShape<L, E>::TWSIZE;   // the twiddle table's copy
   static constexpr size_t SMEM = NSLOT * BUF + TW + 2 * NSLOT * sizeof(uint64_t) + NSLOT * sizeof(ChainSlot);
-  // resident CTAs per SM the register budget is held to (what shared memory allows at L = 512)
-  static constexpr int MIN_BLOCKS = L <= 512 ? (NSLOT == 2 ? 3 : 2) : 1;
+  // resident CTAs per SM the register budget is held to: what shared memory
+  // allows at L = 512, and below, but for the forward transforms with 32
+  // values per thread, which would spill
+  static constexpr int min_blocks(bool fwd) {
+    return L == 1024 ? 1 : L == 512 || (E == 32 && fwd) ? (NSLOT == 2 ? 3 : 2) : L == 256 ? (NSLOT == 2 ? 6 : 4)
+                                                                                : (NSLOT == 2 ? 10 : 8);
+  }
   // the consumers' named barrier counts whole warps
   static_assert(CONSUMERS % 32 == 0, "consumer threads must be whole warps");
 };
@@ -98,24 +114,24 @@ template <int L, int NSLOT = 2> struct ChainTile {
 // (the kernel keeps a copy of the twiddle table in shared memory: its data
 // slots take most of the SM's shared memory, leaving little L1 for the
 // table's global reads)
-template <int L, int IC, int LD, int ST, class TS, bool INV>
+template <int L, int E, int IC, int LD, int ST, class TS, bool INV>
 struct ChainTmaCtx : AxisTmaCtx<L, IC, LD, ST, TS, INV> {
-  static constexpr int kBarThreads = ChainTile<L>::CONSUMERS;
+  static constexpr int kBarThreads = ChainTile<L, E>::CONSUMERS;
   static constexpr bool kTwShared = true;
 };
-template <int L, int IC, class TS>
+template <int L, int E, int IC, class TS>
 struct ChainTmaPairCtx : AxisTmaPairCtx<L, IC, TS> {
-  static constexpr int kBarThreads = ChainTile<L>::CONSUMERS;
+  static constexpr int kBarThreads = ChainTile<L, E>::CONSUMERS;
   static constexpr bool kTwShared = true;
   __device__ __forceinline__ void store(int l, const float2 (&x)[1]) const {
-    this->smem[padE<kChainE>(l) * IC + this->c] = x[0];
+    this->smem[padE<E>(l) * IC + this->c] = x[0];
   }
 };
 // y inverse of the inverse chain: stores the intermediate with an L2
 // evict-last policy (it is read back within microseconds, then dropped)
-template <int L, int IC, class TS>
+template <int L, int E, int IC, class TS>
 struct ChainMidCtx : AxisTmaCtx<L, IC, kLoadCpx, kStoreCpx, TS, true> {
-  static constexpr int kBarThreads = ChainTile<L>::CONSUMERS;
+  static constexpr int kBarThreads = ChainTile<L, E>::CONSUMERS;
   static constexpr bool kTwShared = true;
   static constexpr bool kLoadRow = sizeof(TS) == 8;   // places in psi_pos order
   uint64_t keep;
@@ -139,8 +155,8 @@ struct ChainMidCtx : AxisTmaCtx<L, IC, kLoadCpx, kStoreCpx, TS, true> {
 
 // the second transform of either chain: its output is not read again while
 // the chain runs, so it is stored evict-first and leaves L2 to the intermediate
-template <int L, int IC, int ST, class TS, bool INV>
-struct ChainOutCtx : ChainTmaCtx<L, IC, kLoadCpx, ST, TS, INV> {
+template <int L, int E, int IC, int ST, class TS, bool INV>
+struct ChainOutCtx : ChainTmaCtx<L, E, IC, kLoadCpx, ST, TS, INV> {
   uint64_t stream;
   __device__ __forceinline__ void store(int l, const float2 (&x)[1]) const {
     float2 v = x[0];
@@ -157,8 +173,8 @@ struct ChainOutCtx : ChainTmaCtx<L, IC, kLoadCpx, ST, TS, INV> {
   }
 };
 
-template <int L> __device__ __forceinline__ void consumer_sync() {
-  asm volatile("bar.sync 1, %0;" ::"r"(ChainTile<L>::CONSUMERS) : "memory");
+template <int CONSUMERS> __device__ __forceinline__ void consumer_sync() {
+  asm volatile("bar.sync 1, %0;" ::"r"(CONSUMERS) : "memory");
 }
 
 // common fields of a staged complex sub-tile's transform context
@@ -192,12 +208,13 @@ __device__ __forceinline__ void chain_ctx(Ctx& ctx, float2* slot, const float2* 
 // issued before (by this or another CTA) and need nothing but their
 // consumers: the kernel cannot deadlock, and every wait is bounded.
 template <int L, class TS, bool kFwd, int ST, int NSLOT>
-__global__ void __launch_bounds__(ChainTile<L, NSLOT>::THREADS, ChainTile<L, NSLOT>::MIN_BLOCKS)
+__global__ void __launch_bounds__(ChainTile<L, chain_e<L, TS>(), NSLOT>::THREADS,
+                                  ChainTile<L, chain_e<L, TS>(), NSLOT>::min_blocks(kFwd))
 fk_chain_kernel(const __grid_constant__ CUtensorMap map, const FkChainParams p) {
-  using T = ChainTile<L, NSLOT>;
+  constexpr int E = chain_e<L, TS>();
+  using T = ChainTile<L, E, NSLOT>;
   using TR = typename RealOf<TS>::T;
   constexpr int IC = kChainIC;
-  constexpr int E = kChainE;
   constexpr int TPC = L / E;
   extern __shared__ __align__(128) unsigned char cs[];
   auto buf = [&](int slot) { return reinterpret_cast<float2*>(cs + slot * T::BUF); };
@@ -224,7 +241,8 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map, const FkChainParams p) 
     }
     mbar_fence_init();
   }
-  for (int i = threadIdx.x; i < FftShape<L, kChainE>::TWSIZE; i += T::THREADS) tw[i] = __ldg(p.tw + i);
+  const float2* tw_src = E == 32 ? p.tw32 : p.tw;
+  for (int i = threadIdx.x; i < FftShape<L, E>::TWSIZE; i += T::THREADS) tw[i] = __ldg(tw_src + i);
   __syncthreads();
   pdl_wait();
 
@@ -328,7 +346,7 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map, const FkChainParams p) 
       if (kFwd && !it.second) {
         // x forward of wall row y = idx: 16 real columns t0 + c, t0 + c + 8
         const int t0 = it.chunk * kChainCols;
-        ChainTmaPairCtx<L, IC, TS> ctx;
+        ChainTmaPairCtx<L, E, IC, TS> ctx;
         ctx.tile = reinterpret_cast<const TR*>(buf(slot));
         ctx.smem = buf(slot);
         ctx.tw = tw;
@@ -336,8 +354,8 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map, const FkChainParams p) 
         ctx.c = c;
         ctx.m0 = p.t_scale != 0.f ? ldm * (float)(t0 + c) * p.t_scale : ldm;
         ctx.m1 = p.t_scale != 0.f ? ldm * (float)(t0 + c + IC) * p.t_scale : ldm;
-        fftn_run<L, 1, true, false, ChainTmaPairCtx<L, IC, TS>, E>(ctx, j0);
-        consumer_sync<L>();
+        fftn_run<L, 1, true, false, ChainTmaPairCtx<L, E, IC, TS>, E>(ctx, j0);
+        consumer_sync<T::CONSUMERS>();
         // split the two real columns: X_c[k] = (Z[k] + conj Z[L-k]) / 2,
         // X_{c+8}[k] = (Z[k] - conj Z[L-k]) / (2i), k in [0, L/2]
         const float h = 0.5f * p.s1;
@@ -358,7 +376,7 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map, const FkChainParams p) 
       } else if (kFwd) {
         // y forward of kx = idx: rows y < b, all L outputs (stored evict-first:
         // the spectrum is read by the next stage, after this one)
-        ChainOutCtx<L, IC, kStoreCpx, TS, false> ctx;
+        ChainOutCtx<L, E, IC, kStoreCpx, TS, false> ctx;
         chain_ctx(ctx, buf(slot), tw, c);
         ctx.stream = once;
         ctx.out = p.out;
@@ -369,10 +387,10 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map, const FkChainParams p) 
         ctx.L_in = p.b;
         ctx.L_out = L;
         ctx.stmul = p.s2;
-        fftn_run<L, 1, true, false, ChainOutCtx<L, IC, kStoreCpx, TS, false>, E>(ctx, j0);
+        fftn_run<L, 1, true, false, ChainOutCtx<L, E, IC, kStoreCpx, TS, false>, E>(ctx, j0);
       } else if (!it.second) {
         // y inverse of kx = idx: keep y < b
-        ChainMidCtx<L, IC, TS> ctx;
+        ChainMidCtx<L, E, IC, TS> ctx;
         chain_ctx(ctx, buf(slot), tw, c);
         ctx.keep = keep;
         ctx.out = p.mid;
@@ -383,10 +401,10 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map, const FkChainParams p) 
         ctx.L_in = L;
         ctx.L_out = p.b;
         ctx.stmul = p.s1;
-        fftn_run<L, 1, false, true, ChainMidCtx<L, IC, TS>, E>(ctx, j0);
+        fftn_run<L, 1, false, true, ChainMidCtx<L, E, IC, TS>, E>(ctx, j0);
       } else {
         // x inverse of wall row y = idx: keep x < a, |.|^2 (or complex)
-        ChainOutCtx<L, IC, ST, TS, true> ctx;
+        ChainOutCtx<L, E, IC, ST, TS, true> ctx;
         chain_ctx(ctx, buf(slot), tw, c);
         ctx.stream = once;
         ctx.out = p.out;
@@ -397,13 +415,13 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map, const FkChainParams p) 
         ctx.L_in = L;
         ctx.L_out = p.a;
         ctx.stmul = p.s2 * std_;
-        fftn_run<L, 1, false, true, ChainOutCtx<L, IC, ST, TS, true>, E>(ctx, j0);
+        fftn_run<L, 1, false, true, ChainOutCtx<L, E, IC, ST, TS, true>, E>(ctx, j0);
       }
     }
     // no consumer touches the slot any more: order the shared-memory
     // accesses before the next copy into it and release it; a finished
     // first-transform item also publishes its stores
-    consumer_sync<L>();
+    consumer_sync<T::CONSUMERS>();
     if (threadIdx.x == 0) {
       fence_proxy_async_smem();
       mbar_arrive(&empty[slot]);
@@ -417,7 +435,7 @@ fk_chain_kernel(const __grid_constant__ CUtensorMap map, const FkChainParams p) 
 
 template <int L, class TS, int NSLOT>
 cudaError_t launch_fk_chain_one(const FkChainLaunch& l, cudaStream_t s) {
-  using T = ChainTile<L, NSLOT>;
+  using T = ChainTile<L, chain_e<L, TS>(), NSLOT>;
   const FkChainParams& p = l.p;
   void (*k)(const __grid_constant__ CUtensorMap, const FkChainParams) =
       l.fwd ? fk_chain_kernel<L, TS, true, kStoreCpx, NSLOT>

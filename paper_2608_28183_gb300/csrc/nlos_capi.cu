@@ -853,7 +853,8 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
   bool after = false;   // another kernel of this call precedes
   if (part != 2 && sync_bytes) NLOS_CU(cudaMemsetAsync(sync_inv, 0, sync_bytes, s), "fk chain counters");
   if (p->fused || p->fused_inv) {
-    ch.tw = p->tw32[(int)Lx];   // radix-32 schedule
+    ch.tw = p->tw[(int)Lx];
+    ch.tw32 = p->tw32[(int)Lx];
     ch.a = (int)a;
     ch.b = (int)b;
     ch.n = (int)n;

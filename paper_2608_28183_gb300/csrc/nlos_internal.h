@@ -157,7 +157,8 @@ struct FkChainParams {
   const void* in;
   void* mid;
   void* out;
-  const float2* tw;            // twiddles for L
+  const float2* tw;            // twiddles for L, radix-16 schedule
+  const float2* tw32;          // radix-32 schedule
   int a, b, n, L;
   int nchunks;                 // n / 16
   int lag;                     // chunks between a chunk's first- and second-transform tickets (set by the launcher)
