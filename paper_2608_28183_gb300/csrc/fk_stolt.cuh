@@ -59,31 +59,37 @@ __device__ __forceinline__ StoltCoord stolt_coord(float Ahi, float Alo, int m, i
 // about 1.5e-8 / mu). S then takes one exact sum instead of two, and the
 // weight's rollover at an integer one floor instead of two branches.
 struct StoltSplitA {
-  int Ai;
+  float Ai;   // an integer, at most 2^24
   float Af;
 };
 __device__ __forceinline__ StoltSplitA stolt_split_a(float Ahi, float Alo) {
   // sources with A >= 2^24 lie outside every spectrum: A is clamped to
   // exactly 2^24 (and the sum stays positive and in range); so is a NaN
-  if (!(Ahi < 16777216.f)) return {16777216, 0.f};
-  const int Ai = (int)Ahi;   // floor: A >= 0; Ahi - Ai is exact
-  return {Ai, (Ahi - (float)Ai) + Alo};
+  if (!(Ahi < 16777216.f)) return {16777216.f, 0.f};
+  const float Ai = floorf(Ahi);   // A >= 0; Ahi - Ai is exact
+  return {Ai, (Ahi - Ai) + Alo};
 }
-// m >= 1, fm = (float)m
-__device__ __forceinline__ StoltCoord stolt_coord_split(const StoltSplitA& a, int m, float fm, int n) {
+// floor(x), |x| < 2^22, without the conversion unit (whose quarter rate the
+// coordinate's seven conversions and roundings took a quarter of the stage's
+// time in): 1.5 * 2^23 + x rounded down has the floor in its low bits
+constexpr float kFloorBias = 12582912.f;
+constexpr int kFloorBits = 0x4B400000;        // the bias as an integer
+__device__ __forceinline__ float floor_biased(float x) { return __fadd_rd(x, kFloorBias); }
+// m >= 1, m <= 4096, fm = (float)m
+__device__ __forceinline__ StoltCoord stolt_coord_split(const StoltSplitA& a, float fm, int n) {
   StoltCoord c;
-  const float sx = (float)(a.Ai + m * m);
+  const float sx = fmaf(fm, fm, a.Ai);        // Ai + m^2, rounded once
   const float sh = sx + a.Af;                 // |sx| >= 1 >= |Af|: fast two-sum
   const float sl = a.Af - (sh - sx);
   const float rs = rsqrtf(sh);
   const float y0 = sh * rs;
   const float res = fmaf(-y0, y0, sh) + sl;   // S - y0^2
   const float mlo = res * (0.5f * rs);        // mu = y0 + mlo
-  int k0 = (int)floorf(y0);
-  float al = (y0 - (float)k0) + mlo;
-  const float roll = floorf(al);              // -1, 0 or 1: y0 is within a few ulp of mu
-  k0 += (int)roll;
-  al -= roll;
+  const float t0 = floor_biased(y0);
+  float al = (y0 - (t0 - kFloorBias)) + mlo;
+  const float t1 = floor_biased(al);          // -1, 0 or 1: y0 is within a few ulp of mu
+  al -= t1 - kFloorBias;
+  const int k0 = __float_as_int(t0) + (__float_as_int(t1) - 2 * kFloorBits);
   c.valid = (k0 < n - 1) || (k0 == n - 1 && al == 0.f);
   c.k0 = k0;
   c.k1 = k0 + 1;

@@ -70,7 +70,11 @@ struct FkLiteFwdCtx {
     }
   }
   __device__ __forceinline__ float2* sm(int) const { return U; }
-  __device__ __forceinline__ void store(int l, const float2 (&x)[1]) const { U[l] = x[0]; }
+  // U[L] repeats U[0]: the gather of the negative frequencies, U[L - k], needs no wrap
+  __device__ __forceinline__ void store(int l, const float2 (&x)[1]) const {
+    U[l] = x[0];
+    if (l == 0) U[L] = x[0];
+  }
 };
 
 // E: values per thread of the transforms (16: radix-16 passes, 32: radix-32)
@@ -176,17 +180,19 @@ __global__ void __launch_bounds__(FkLiteTile<L, PPC, E>::THREADS, FkLiteTile<L, 
   for (int m = m0; m < L / 2; m += S::TPC, fm += (float)S::TPC) {
     float2 d = make_float2(0.f, 0.f), e = d;
     if (m >= 1) {
-      const StoltCoord c = stolt_coord_split(As, m, fm, L / 2);
+      const StoltCoord c = stolt_coord_split(As, fm, L / 2);
       if (c.valid) {
         // k0 + 1 <= L/2 is in the spectrum; at k0 = L/2 - 1 its weight alpha is 0
-        const int k1 = c.k1;
-        const float2 u0 = U[c.k0], u1 = U[k1];
-        const float2 w0 = U[(L - c.k0) & (L - 1)], w1 = U[(L - k1) & (L - 1)];
+        const float2* up = U + c.k0;
+        const float2* un = U + (L - c.k0);
+        const float2 u0 = up[0], u1 = up[1], w0 = un[0], w1 = un[-1];
         // (1 - alpha) u0 + alpha u1, times the Jacobian m/mu and the scale
         const float b1 = c.jac * st * c.alpha;
         const float b0 = fmaf(c.jac, st, -b1);
-        d = make_float2(fmaf(b1, u1.x, b0 * u0.x), fmaf(b1, u1.y, b0 * u0.y));
-        e = make_float2(fmaf(b1, w1.x, b0 * w0.x), -fmaf(b1, w1.y, b0 * w0.y));
+        const float2 b0p = make_float2(b0, b0), b1p = make_float2(b1, b1);
+        d = __ffma2_rn(b1p, u1, __fmul2_rn(b0p, u0));
+        e = __ffma2_rn(b1p, w1, __fmul2_rn(b0p, w0));
+        e.y = -e.y;
       }
     }
     if (!kStep) om = (m >> 3) * s8 + (m & 7);
