@@ -825,10 +825,22 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
   int sid = 0;
   if (part != 2) NLOS_MARK(p, s, -1);
   const float ramp = 1.0f / (float)(n - 1);
+  // chunk counters of the fused forward at off_sync, those of the fused inverse
+  // before it, short of the last 256 bytes of the scale partials' area (whose last
+  // word counts the volume scale's CTAs): one clear for all, ahead of the
+  // first kernel
+  static_assert(kScalePartials * sizeof(float) >= 152 * 4 * sizeof(float) + 256 + 4 * 512, "partials, counters");
+  const size_t inv_sync_bytes = p->fused_inv ? align256(sizeof(int) * (size_t)(1 + p->zcols / 16)) + 256 : 0;
+  int* sync = reinterpret_cast<int*>(ws + p->off_sync);
+  int* sync_inv = reinterpret_cast<int*>(ws + p->off_sync - inv_sync_bytes);
+  const size_t sync_bytes = inv_sync_bytes + (p->fused ? sizeof(int) * (size_t)(1 + n / 16) : 0);
+  if (part != 2 && sync_bytes) NLOS_CU(cudaMemsetAsync(sync_inv, 0, sync_bytes, s), "fk chain counters");
+  bool after = false;   // another kernel of this call precedes
   if (st != kF32) {
     NLOS_CU(launch_volume_scale(H, a * b * n, (int)n, 1.0f / (float)(n - 1), st, kVolumeTarget,
-                                reinterpret_cast<float*>(ws + p->off_part), kScalePartials, scal, s),
+                                reinterpret_cast<float*>(ws + p->off_part), kScalePartials, scal, inv_sync_bytes > 0, s),
             "volume scale");
+    after = true;
     NLOS_MARK(p, s, sid++);
     s_in = scal;
     inv_s = scal + 1;
@@ -842,16 +854,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
   const bool cpx = p->d.output == NLOS_OUT_COMPLEX;
   const float fscale = (float)(cpx ? 1.0 / (N * gprod) : 1.0 / (N * N * gprod * gprod));
   FkChainParams ch{};
-  // chunk counters of the fused forward at off_sync, those of the fused inverse
-  // in the 256-byte steps before it (the scale partials' end, free once the
-  // volume scale is known): one clear for both, ahead of the first stage
-  int* sync = reinterpret_cast<int*>(ws + p->off_sync);
-  const size_t inv_sync_bytes = p->fused_inv ? align256(sizeof(int) * (size_t)(1 + p->zcols / 16)) : 0;
-  int* sync_inv = reinterpret_cast<int*>(ws + p->off_sync - inv_sync_bytes);
-  const size_t sync_bytes = inv_sync_bytes + (p->fused ? sizeof(int) * (size_t)(1 + n / 16) : 0);
   const size_t rb = real_bytes(st);
-  bool after = false;   // another kernel of this call precedes
-  if (part != 2 && sync_bytes) NLOS_CU(cudaMemsetAsync(sync_inv, 0, sync_bytes, s), "fk chain counters");
   if (p->fused || p->fused_inv) {
     ch.tw = p->tw[(int)Lx];
     ch.tw32 = p->tw32[(int)Lx];
@@ -890,6 +893,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
     if (!encode_3d(&c.map, H, rb, (unsigned long long)(b * n), a, 1, b * n * rb, a * b * n * rb, 16,
                    (unsigned)std::min<long long>(a, 256), false))
       return fail(NLOS_ERR_CUDA, "fk xy-forward: tensor map encoding failed");
+    c.after = after;
     NLOS_CU(launch_fk_chain(c, st, s), "fk xy-forward");
     after = true;
     NLOS_MARK(p, s, sid++);
@@ -907,6 +911,7 @@ nlos_status_t run_fk(nlos_plan_s* p, const void* H, void* vol, char* ws, cudaStr
   l.err = err;
   attach_tmap(l);
   set_extents(l, a * b * n, ws_extent(p, 0));
+  l.after = after;
   NLOS_CU(launch_axis_fft(l, s), "fk x-forward");
   after = true;
   NLOS_MARK(p, s, sid++);
@@ -1080,7 +1085,7 @@ nlos_status_t run_pf(nlos_plan_s* p, const void* H, const void* P_in, void* vol,
   NLOS_MARK(p, s, -1);
   if (st != kF32 && !P_in && !G0) {
     NLOS_CU(launch_volume_scale(H, a * b * n, (int)n, 0.0f, st, kVolumeTarget,
-                                reinterpret_cast<float*>(ws + p->off_part), kScalePartials, scal, s),
+                                reinterpret_cast<float*>(ws + p->off_part), kScalePartials, scal, false, s),
             "volume scale");
     NLOS_MARK(p, s, sid++);
     s_in = scal;

@@ -374,8 +374,9 @@ cudaError_t launch_pf_dense(const PfDenseParams& p, cudaStream_t s);
 
 // Per-volume scale for reduced-precision storage: out[0] = target / ||u||_2,
 // out[1] = 1 / out[0], out[2] = 1 / out[0]^2, where u = H * (t % n) * t_scale (t_scale = 0: no ramp).
+// `cleared`: the caller has zeroed the last of the partials, the CTAs' counter.
 cudaError_t launch_volume_scale(const void* H, long long count, int n, float t_scale, int storage,
-                                float target, float* partial, int npartial, float* out,
+                                float target, float* partial, int npartial, float* out, bool cleared,
                                 cudaStream_t s);
 
 }  // namespace nlos

@@ -719,7 +719,7 @@ __global__ void sumsq_partial_kernel(const TR* H, long long count, int n, float 
 }
 
 cudaError_t launch_volume_scale(const void* H, long long count, int n, float t_scale, int storage,
-                                float target, float* partial, int npartial, float* out, cudaStream_t s) {
+                                float target, float* partial, int npartial, float* out, bool cleared, cudaStream_t s) {
   // four CTAs per SM (enough bytes in flight with 16-byte loads); the count
   // of partials only changes the summation tree, not determinism. The last
   // partial slot holds the CTAs' completion counter.
@@ -727,7 +727,7 @@ cudaError_t launch_volume_scale(const void* H, long long count, int n, float t_s
   if (blocks < 1) return cudaErrorInvalidValue;
   unsigned* counter = reinterpret_cast<unsigned*>(partial + npartial - 1);
   // a caller's workspace may hold anything there on its first use
-  cudaError_t e0 = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
+  cudaError_t e0 = cleared ? cudaSuccess : cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
   if (e0 != cudaSuccess) return e0;
   const bool vec = (reinterpret_cast<uintptr_t>(H) & 15) == 0;
   switch (storage) {

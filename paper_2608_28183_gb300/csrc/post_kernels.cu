@@ -17,12 +17,16 @@ namespace {
 
 using nlos::set_error;
 
-// one warp per (x, y) pencil, lanes stride along the contiguous depth axis
+// one warp per (x, y) pencil, lanes stride along the contiguous depth axis. The
+// pencils are taken from the last to the first: a volume that was just written
+// from the first on has its end in L2 (after a coherence merge of 4 x 256 MB
+// into 134 MB: 3 us of 23).
 __global__ void max_image_kernel(const float* __restrict__ v, long long nxy, int nz, int take_sqrt,
                                  float* __restrict__ img) {
-  const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (w >= nxy) return;
+  if (r >= nxy) return;
+  const long long w = nxy - 1 - r;
   const float* p = v + w * nz;
   float m = -INFINITY;
   for (int z = lane; z < nz; z += 32) m = fmaxf(m, p[z]);
@@ -189,16 +193,15 @@ __global__ void dda_vec_kernel(const __grid_constant__ FramePtrs fr, int nw, lon
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
+// One pass per thread, as many CTAs as that takes: the block scheduler keeps the
+// loads of the frames coming, where persistent CTAs (eight of 256 threads per
+// SM) wait out each iteration's latency. Coherence merge of four
+// 256x256x512 volumes: 218 us persistent, 185 us so (1.208 GB, 6.5 TB/s), the
+// same with 256 threads, 189 with 512.
+constexpr int kPostThreads = 128;
 int grid_for(long long work) {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (sms <= 0) sms = 1;
-  }
-  const long long want = (work + 255) / 256;
-  return (int)std::max<long long>(1, std::min<long long>(want, (long long)sms * 8));
+  const long long want = (work + kPostThreads - 1) / kPostThreads;
+  return (int)std::max<long long>(1, std::min<long long>(want, 0x7fffffffLL));
 }
 
 nlos_status_t launch_status(const char* what) {
@@ -246,10 +249,10 @@ nlos_status_t nlos_coherence_merge(const void* const* frames, int nw, long long 
   cudaGetLastError();
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (vec)
-    coherence_vec_kernel<<<grid_for(count / 2), 256, 0, s>>>(fp, nw, count / 2, eps, reinterpret_cast<float2*>(merged),
+    coherence_vec_kernel<<<grid_for(count / 2), kPostThreads, 0, s>>>(fp, nw, count / 2, eps, reinterpret_cast<float2*>(merged),
                                                             reinterpret_cast<float2*>(coherence));
   else
-    coherence_kernel<<<grid_for(count), 256, 0, s>>>(fp, nw, count, eps, merged, coherence);
+    coherence_kernel<<<grid_for(count), kPostThreads, 0, s>>>(fp, nw, count, eps, merged, coherence);
   return launch_status("coherence merge");
 }
 
@@ -266,9 +269,9 @@ nlos_status_t nlos_dda(const float* const* frames, int nw, long long nxy, int nz
   cudaGetLastError();
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (vec)
-    dda_vec_kernel<<<grid_for(nxy * (nz / 4)), 256, 0, s>>>(fp, nw, nxy, nz, reinterpret_cast<float4*>(out));
+    dda_vec_kernel<<<grid_for(nxy * (nz / 4)), kPostThreads, 0, s>>>(fp, nw, nxy, nz, reinterpret_cast<float4*>(out));
   else
-    dda_kernel<<<grid_for(nxy * nz), 256, 0, s>>>(fp, nw, nxy, nz, out);
+    dda_kernel<<<grid_for(nxy * nz), kPostThreads, 0, s>>>(fp, nw, nxy, nz, out);
   return launch_status("depth-dependent average");
 }
 
