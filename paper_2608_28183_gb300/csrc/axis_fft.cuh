@@ -2,7 +2,7 @@
 // [outer][L][inner] array with `inner` contiguous. A CTA owns IC consecutive
 // inner columns of one outer slice, so every global access is a run of IC
 // consecutive elements (coalesced); the IC transforms run side by side with
-// TPC = L/16 threads each, exchanging through shared memory laid out as
+// TPC = L/16 (L/32) threads each, exchanging through shared memory laid out as
 // [padded row][IC].
 #pragma once
 #include <algorithm>
@@ -31,11 +31,30 @@ inline cudaError_t axis_report(const char* path, int L, int ic, int threads, siz
   return e;
 }
 
-template <int L, int IC_> struct AxisTile {
+// Values per thread. 32 at 512 points where fft_joined_run saves an exchange
+// and the time: the TMA-staged forward transforms (zero-padded upper half), and
+// the staged cropped inverses at 16 columns. Half the threads hide less of the
+// memory's latency, so the transforms that load directly, or whose tiles are
+// full and narrow, keep 16. Measured per pass at the best tile (16 -> 32
+// values): phasor field 256x256x512 f16 y 47 -> 44 us, x 90 -> 80, y inverse at
+// 16 columns 84 -> 68 (74 at 8 columns with 16 values), x inverse 43 -> 57;
+// f-k 190x190x3002 float32 x pairs 423 -> 404, y with direct loads 862 -> 1023.
+constexpr int axis_e(int L, int ic, bool staged, bool half_in, bool half_out) {
+  return L == 512 && staged && (half_in || (half_out && ic == 16)) ? 32 : 16;
+}
+template <int L, int IC_, int E_ = 16> struct AxisTile {
   static constexpr int IC = IC_;
-  static constexpr int THREADS = IC * (L / 16);
+  static constexpr int E = E_;
+  static constexpr int TPC = L / E;
+  static constexpr int THREADS = IC * TPC;
   static constexpr size_t SMEM = (L > 16) ? sizeof(float2) * FftShape<L>::SMEM * IC : 0;
 };
+
+template <int L, int E, bool kHalfIn, bool kHalfOut, class Ctx>
+__device__ __forceinline__ void axis_run(Ctx& ctx, const int j0) {
+  if constexpr (E == 32) fft_joined_run<L, kHalfIn, kHalfOut>(ctx, j0);
+  else fftn_run<L, 1, kHalfIn, kHalfOut>(ctx, j0);
+}
 
 // INV: inverse transform (e^{+i})
 template <int L, int IC_, int LD, int ST, class TS, bool INV>
@@ -44,6 +63,7 @@ struct AxisCtx {
   static constexpr int IC = IC_;
   static constexpr int SSTRIDE = IC;
   static constexpr bool kSmemInput = false;
+  static constexpr bool kSmemOutput = false;
   static constexpr bool kInverse = INV;
   const void* in;
   void* out;
@@ -121,7 +141,7 @@ template <int L, int IC, class TS, bool kHalfIn>
 __global__ void __launch_bounds__(AxisTile<L, IC>::THREADS)
 axis_fft_realpair_kernel(const AxisParams p) {
   extern __shared__ float2 pair_sm[];
-  constexpr int TPC = L / 16;
+  constexpr int TPC = AxisTile<L, IC>::TPC;
   pdl_trigger();
   pdl_wait();
   const int c = threadIdx.x % IC;
@@ -230,21 +250,22 @@ struct AxisTmaCtx : AxisCtx<L, IC, LD, ST, TS, INV> {
   }
 };
 
-template <int L, int IC, int LD, class TS> struct AxisTmaTile {
+template <int L, int IC, int LD, class TS, int E> struct AxisTmaTile {
   using TR = typename RealOf<TS>::T;
   static constexpr size_t ELEM = LD == kLoadReal ? sizeof(TR) : sizeof(TS);
   static constexpr size_t BUF = sizeof(float2) * FftShape<L>::SMEM * IC;   // bytes per buffer (multiple of 128)
   static constexpr size_t SMEM = 2 * BUF + 2 * sizeof(uint64_t);
-  static constexpr int THREADS = IC * (L / 16);
+  static constexpr int THREADS = AxisTile<L, IC, E>::THREADS;
 };
 
 constexpr int kTmaWaitLimit = 1 << 21;   // polls; each may suspend briefly, ~1 s in all
 
 template <int L, int IC, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut, bool INV>
-__global__ void __launch_bounds__(AxisTile<L, IC>::THREADS)
+__global__ void __launch_bounds__(AxisTile<L, IC, axis_e(L, IC, true, kHalfIn, kHalfOut)>::THREADS)
 axis_fft_tma_kernel(const __grid_constant__ CUtensorMap tmap, const AxisParams p, const int tiles_inner,
                     const long long ntiles, int* err) {
-  using T = AxisTmaTile<L, IC, LD, TS>;
+  constexpr int E = axis_e(L, IC, true, kHalfIn, kHalfOut);
+  using T = AxisTmaTile<L, IC, LD, TS, E>;
   extern __shared__ __align__(128) unsigned char tma_sm[];
   auto buf = [&](int slot) { return reinterpret_cast<float2*>(tma_sm + slot * T::BUF); };
   uint64_t* bar = reinterpret_cast<uint64_t*>(tma_sm + 2 * T::BUF);
@@ -309,14 +330,14 @@ axis_fft_tma_kernel(const __grid_constant__ CUtensorMap tmap, const AxisParams p
     ctx.stmul = stmul;
     ctx.out_n = p.out_n;
     ctx.err = p.err;
-    fftn_run<L, 1, kHalfIn, kHalfOut>(ctx, j0);
+    axis_run<L, E, kHalfIn, kHalfOut>(ctx, j0);
     __syncthreads();   // the buffer is free before the next issue into it
   }
 }
 
 template <int L, int IC, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut, bool INV>
 cudaError_t launch_axis_tma(const AxisLaunch& l, cudaStream_t s) {
-  using T = AxisTmaTile<L, IC, LD, TS>;
+  using T = AxisTmaTile<L, IC, LD, TS, axis_e(L, IC, true, kHalfIn, kHalfOut)>;
   auto k = axis_fft_tma_kernel<L, IC, LD, ST, TS, kHalfIn, kHalfOut, INV>;
   static int blocks_per_sm = 0;
   static int sms = 0;
@@ -349,6 +370,7 @@ struct AxisTmaPairCtx {
   using TR = typename RealOf<TS>::T;
   static constexpr int SSTRIDE = IC;
   static constexpr bool kSmemInput = true;
+  static constexpr bool kSmemOutput = true;
   const TR* tile;       // staged tile, [row][2 IC] reals
   float2* smem;
   const float2* tw;
@@ -365,12 +387,13 @@ struct AxisTmaPairCtx {
 };
 
 template <int L, int IC, class TS, bool kHalfIn>
-__global__ void __launch_bounds__(AxisTile<L, IC>::THREADS)
+__global__ void __launch_bounds__(AxisTile<L, IC, axis_e(L, IC, true, kHalfIn, false)>::THREADS)
 axis_fft_tma_pair_kernel(const __grid_constant__ CUtensorMap tmap, const AxisParams p, const int tiles_inner,
                          const long long ntiles, int* err) {
   using TR = typename RealOf<TS>::T;
   constexpr size_t BUF = sizeof(float2) * FftShape<L>::SMEM * IC;
-  constexpr int TPC = L / 16;
+  constexpr int E = axis_e(L, IC, true, kHalfIn, false);
+  constexpr int TPC = AxisTile<L, IC, E>::TPC;
   extern __shared__ __align__(128) unsigned char tp_sm[];
   auto buf = [&](int slot) { return reinterpret_cast<float2*>(tp_sm + slot * BUF); };
   uint64_t* bar = reinterpret_cast<uint64_t*>(tp_sm + 2 * BUF);
@@ -424,7 +447,7 @@ axis_fft_tma_pair_kernel(const __grid_constant__ CUtensorMap tmap, const AxisPar
     ctx.c = c;
     ctx.m0 = ldmul * (p.t_len > 0 ? (float)(int)(ii0 % p.t_len) * p.t_scale : 1.0f);
     ctx.m1 = ldmul * (p.t_len > 0 ? (float)(int)(ii1 % p.t_len) * p.t_scale : 1.0f);
-    fftn_run<L, 1, kHalfIn, false>(ctx, j0);
+    axis_run<L, E, kHalfIn, false>(ctx, j0);
     __syncthreads();
     const float2* z = buf(slot);
     const bool v0 = ii0 < p.inner, v1 = ii1 < p.inner;
@@ -443,7 +466,7 @@ template <int L, int IC, class TS, bool kHalfIn>
 cudaError_t launch_axis_tma_pair(const AxisLaunch& l, cudaStream_t s) {
   constexpr size_t BUF = sizeof(float2) * FftShape<L>::SMEM * IC;
   constexpr size_t SMEM = 2 * BUF + 2 * sizeof(uint64_t);
-  constexpr int THREADS = AxisTile<L, IC>::THREADS;
+  constexpr int THREADS = AxisTile<L, IC, axis_e(L, IC, true, kHalfIn, false)>::THREADS;
   auto k = axis_fft_tma_pair_kernel<L, IC, TS, kHalfIn>;
   static int blocks_per_sm = 0;
   static int sms = 0;

@@ -375,6 +375,75 @@ __device__ __forceinline__ void fftn_run(Ctx& ctx, const int j0) {
   fftn_passes<L, NT, kHalfIn, kHalfOut, 0, Ctx, E>(ctx, j0, v);
 }
 
+// A transform of L = 2 * 16^2 points with both radix-16 butterflies that its
+// closing radix-2 pass joins in one thread (TPC = L/32 threads, 32 values each):
+// butterflies j and j + 16 of the second pass give elements j + 16 r and
+// 256 + j + 16 r, the pairs of the last, so that pass runs in registers. The
+// arithmetic is that of fftn_run, bit for bit.
+// The strided passes are bound by the shared-memory path: this saves one of
+// the two exchanges (a write, a read and two barriers per value) and half of
+// the second pass's twiddle loads, as j and j + 16 share them.
+// Contexts declare kSmemOutput where store() writes the buffer of the passes.
+template <int L, bool kHalfIn, bool kHalfOut, class Ctx>
+__device__ __forceinline__ void fft_joined_run(Ctx& ctx, const int j0) {
+  using S = FftShape<L>;
+  static_assert(S::NPASS == 3 && S::radix(2) == 2, "two radix-16 passes and a radix-2 pass");
+  constexpr int TPC = L / 32, Q = L / 16, SS = Ctx::SSTRIDE;
+  constexpr bool INV = CtxInverse<Ctx>::value;
+  float2 v[2][16];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      if (kHalfIn && r >= 8) {
+        v[i][r] = make_float2(0.f, 0.f);
+      } else {
+        float2 x[1];
+        ctx.load(j0 + i * TPC + r * Q, x);
+        v[i][r] = x[0];
+      }
+    }
+  if constexpr (Ctx::kSmemInput) fft_sync<Ctx>();
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    if constexpr (kHalfIn) Dft<16, INV>::run_half(v[i]);
+    else Dft<16, INV>::run(v[i]);
+    float2* s = ctx.sm(0) + 17 * (j0 + i * TPC) * SS;   // pad16(16 j + r) = 17 j + r
+#pragma unroll
+    for (int r = 0; r < 16; ++r) s[r * SS] = v[i][r];
+  }
+  fft_sync<Ctx>();
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const float2* s = ctx.sm(0) + pad16(j0 + i * TPC) * SS;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[i][r] = s[r * (Q + Q / 16) * SS];
+  }
+  if constexpr (Ctx::kSmemOutput) fft_sync<Ctx>();
+  static_assert(TPC == 16, "butterflies j and j + TPC share the second pass's twiddles");
+  const float2* tp = ctx.tw + S::twoff(1) + j0;
+#pragma unroll
+  for (int r = 1; r < 16; ++r) {
+    const float2 w = __ldg(tp + r * 16);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) v[i][r] = INV ? cmulc(v[i][r], w) : cmul(v[i][r], w);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) Dft<16, INV>::run(v[i]);
+  const float2* tl = ctx.tw + S::twoff(2) + L / 2 + j0;
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    const float2 w = __ldg(tl + r * 16);
+    const float2 b = INV ? cmulc(v[1][r], w) : cmul(v[1][r], w);
+    const float2 lo[1] = {cadd(v[0][r], b)};
+    ctx.store(j0 + r * 16, lo);
+    if constexpr (!kHalfOut) {
+      const float2 hi[1] = {csub(v[0][r], b)};
+      ctx.store(j0 + r * 16 + L / 2, hi);
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // storage types for complex intermediates and real inputs
 // ---------------------------------------------------------------------------
