@@ -50,29 +50,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Non-blocking probe of the phase with the given parity.
-__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n"
-      " .reg .pred p;\n"
-      " mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n"
-      "}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Spin on the phase with the given parity, at most `limit` probes (for waits
-// expected to be short, where a suspended try_wait would add its wake-up delay).
-__device__ __forceinline__ bool mbar_spin_bounded(uint64_t* bar, uint32_t parity, int limit) {
-  for (int i = 0; i < limit; ++i)
-    if (mbar_test_wait(bar, parity)) return true;
-  return false;
-}
-
 // Wait for the barrier phase `parity` to complete, at most `limit` polls.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, int limit) {
   for (int i = 0; i < limit; ++i)
