@@ -127,7 +127,8 @@ nlos_status_t nlos_plan_create(const nlos_plan_desc_t* desc, nlos_plan_t* out);
  * passes (x forward, y forward, y inverse, x inverse) even where the fused
  * pairs apply (zero-padded f-k with Lx = Ly <= 1024 and nt a multiple of 16:
  * x then y forward in one launch, y then x inverse in another, each pair's
- * intermediate kept in L2). Same arithmetic; for comparison and testing. */
+ * intermediate kept in L2; the inverse pair alone also for other nt in large
+ * float32 plans). Same results up to rounding; for comparison and testing. */
 #define NLOS_PLAN_SEPARATE_AXES 2
 nlos_status_t nlos_plan_create_ex(const nlos_plan_desc_t* desc, int flags, nlos_plan_t* out);
 

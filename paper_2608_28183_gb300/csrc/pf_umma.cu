@@ -28,7 +28,7 @@
 //
 // Two schedules:
 //  * pf_umma_ws_kernel: one persistent CTA per SM, warp-specialised - a
-//    producer warp keeps up to four operand stages in flight, eight warps
+//    producer warp keeps up to four operand stages in flight, sixteen warps
 //    build A, one thread issues the MMAs, four warps run the epilogue - with
 //    two accumulators so a tile's epilogue overlaps the next tile's MMAs; the
 //    tiles left after the last full round are split along the frequency sum
