@@ -15,6 +15,12 @@
 // chain. The first kernel of a call is launched plainly: what precedes it on
 // the stream is not the library's.
 //
+// A chained kernel reads what another kernel of the chain writes with plain
+// loads, never with __ldg or through a const __restrict__ pointer: the
+// non-coherent path is defined only for memory that nothing writes while the
+// kernel is resident, and a chained kernel is resident before its
+// predecessors have finished. Plan tables are constant and may take that path.
+//
 // Kernels of one tile per CTA trigger at their start (the next kernel can
 // then only take SM slots that no CTA of this one is left to fill); persistent
 // ones when they take their last tile.

@@ -191,7 +191,7 @@ struct AChunk {
         constexpr int kV = 4 * sizeof(In) / 16;              // 16-byte loads
         uint4 v[kV];
 #pragma unroll
-        for (int k = 0; k < kV; ++k) v[k] = __ldg(reinterpret_cast<const uint4*>(src) + k);
+        for (int k = 0; k < kV; ++k) v[k] = reinterpret_cast<const uint4*>(src)[k];   // not __ldg: nlos_launch.cuh
 #pragma unroll
         for (int k = 0; k < 4; ++k) h[k] = reinterpret_cast<const In*>(v)[k];
         return;
