@@ -346,6 +346,14 @@ nlos_status_t nlos_selftest_bounds(int* code);
 nlos_status_t nlos_selftest_bounded_wait(int limit, int* code);
 
 /*
+ * Self-test of the bounded wait of a whole warp: one warp waits on a completed
+ * barrier, its first `gave_up` lanes without polls left. *through is the
+ * number of lanes that were let through: 32 if gave_up is 0, else 0 (a warp
+ * gives up as one). Synchronous. Errors: INVALID_ARG, OUT_OF_MEMORY, CUDA.
+ */
+nlos_status_t nlos_selftest_warp_wait(int gave_up, int* through);
+
+/*
  * Stage tracing. While enabled, every reconstruction with this plan records a
  * CUDA event before its first stage and after each stage, on the call's
  * stream (use one stream per plan while profiling).

@@ -258,7 +258,7 @@ template <int L, int IC, int LD, class TS, int E> struct AxisTmaTile {
   static constexpr int THREADS = AxisTile<L, IC, E>::THREADS;
 };
 
-constexpr int kTmaWaitLimit = 1 << 21;   // polls; each may suspend briefly, ~1 s in all
+constexpr int kTmaWaitLimit = 1 << 21;   // polls of a slot's barrier
 
 template <int L, int IC, int LD, int ST, class TS, bool kHalfIn, bool kHalfOut, bool INV>
 __global__ void __launch_bounds__(AxisTile<L, IC, axis_e(L, IC, true, kHalfIn, kHalfOut)>::THREADS)

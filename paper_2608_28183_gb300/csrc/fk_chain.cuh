@@ -51,7 +51,7 @@ template <int L, class TS> constexpr int chain_e() {
   return L <= 256 && sizeof(TS) == 8 ? 16 : 32;
 }
 constexpr int kChainCols = 2 * kChainIC;   // columns (t or z values) per chunk and item
-constexpr int kChainWaitLimit = 1 << 18;   // polls of a chunk counter (~0.1 s with the back-off; below the ~1 s slot waits)
+constexpr int kChainWaitLimit = 1 << 18;   // polls of a chunk counter, under a microsecond each: shorter than the slot waits
 
 __device__ __forceinline__ int ld_acquire(const int* p) {
   int v;

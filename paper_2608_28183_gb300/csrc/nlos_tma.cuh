@@ -50,11 +50,22 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Wait for the barrier phase `parity` to complete, at most `limit` polls.
+// Wait for the barrier phase `parity` to complete, at most `limit` polls. A poll
+// that finds nothing suspends for about 3.8 us (a wait of 200000 polls on a
+// barrier that nothing arrives on took 753 ms): the library's limits of 2^20 and
+// 2^21 polls are about 4 and 8 s.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, int limit) {
   for (int i = 0; i < limit; ++i)
     if (mbar_try_wait(bar, parity)) return true;
   return false;
+}
+
+// The same by a whole warp, with one answer for all of its lanes: false if any
+// lane ran out of polls. For waits that warp-wide instructions follow
+// (__syncwarp, tcgen05.ld): lanes that gave up by themselves would leave the
+// others waiting there without a limit.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int limit) {
+  return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, limit)) != 0;
 }
 
 // 3D tiled TMA load of the box at (c0, c1, c2) into shared memory, completing

@@ -67,7 +67,7 @@ template <int L> struct PfBandTile {
   }
 };
 
-constexpr int kBandWaitLimit = 1 << 21;   // polls of a staged-load barrier (~1 s in all)
+constexpr int kBandWaitLimit = 1 << 21;   // polls of a staged-load barrier
 
 // split the transform of one pencil pair into both pencils' bands (w(f) and
 // the store scale applied) and store them; returns the largest |component| stored

@@ -45,7 +45,7 @@ namespace nlos {
 
 namespace {
 
-constexpr int kWaitLimit = 1 << 20;                    // waits on a barrier, each suspended for a while (~1 s in all)
+constexpr int kWaitLimit = 1 << 20;                    // polls of a barrier
 constexpr uint32_t kSmemBudget = 200 * 1024;           // dynamic shared memory of the stages
 constexpr int kMaxStages = 4;
 
@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
       const int a = j & 1;
       EpiRows<Op> rows;
       epilogue_rows<Op>(p, sg.tile, sg.blk, warp, p.scale * inv_sa, rows);
-      if (!mbar_wait_bounded(&acc_full[a], (j >> 1) & 1, kWaitLimit)) {
+      if (!mbar_wait_warp(&acc_full[a], (j >> 1) & 1, kWaitLimit)) {
         err = 1;
         break;
       }
@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) pf_umma_ws_kernel(const PfUmmaP
         const int g = g0 + u;
         if (g >= total) break;
         const int s = g % kStages, r = g / kStages;
-        if (r >= 1 && !mbar_wait_bounded(&empty[s], (r - 1) & 1, kWaitLimit)) {
+        if (r >= 1 && !mbar_wait_warp(&empty[s], (r - 1) & 1, kWaitLimit)) {
           err = 1;
           break;
         }

@@ -21,7 +21,34 @@ __global__ void bounded_wait_probe_kernel(int limit, int* err) {
   const bool done = nlos::mbar_wait_bounded(&bar, 0, limit);   // no arrival is ever made
   if (!done && threadIdx.x == 0) atomicExch(err, nlos::kDevErrTmaTimeout);
 }
+
+// a completed phase: lanes 0 .. gave_up - 1 have no polls left, the others do
+__global__ void warp_wait_probe_kernel(int gave_up, int* through) {
+  __shared__ uint64_t bar;
+  if (threadIdx.x == 0) {
+    nlos::mbar_init(&bar, 1);
+    nlos::mbar_fence_init();
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(nlos::smem_u32(&bar)) : "memory");
+  }
+  __syncthreads();
+  const bool ok = nlos::mbar_wait_warp(&bar, 0, (int)threadIdx.x < gave_up ? 0 : 1 << 20);
+  if (ok) atomicAdd(through, 1);
+}
 }  // namespace
+
+extern "C" nlos_status_t nlos_selftest_warp_wait(int gave_up, int* through) {
+  using namespace nlos;
+  if (gave_up < 0 || gave_up > 32 || !through)
+    return set_error(NLOS_ERR_INVALID_ARG, "gave_up must be in [0, 32] and through non-NULL");
+  int* d = nullptr;
+  if (cudaMalloc(&d, sizeof(int)) != cudaSuccess) return set_error(NLOS_ERR_OUT_OF_MEMORY, "self-test word");
+  cudaMemset(d, 0, sizeof(int));
+  warp_wait_probe_kernel<<<1, 32>>>(gave_up, d);
+  cudaError_t e = cudaDeviceSynchronize();
+  if (e == cudaSuccess) e = cudaMemcpy(through, d, sizeof *through, cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  return e == cudaSuccess ? NLOS_OK : set_error(NLOS_ERR_CUDA, cudaGetErrorString(e));
+}
 
 extern "C" nlos_status_t nlos_selftest_bounded_wait(int limit, int* code) {
   using namespace nlos;

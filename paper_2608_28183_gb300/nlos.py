@@ -34,6 +34,7 @@ EXPORTED = ["nlos_plan_desc_default", "nlos_plan_create", "nlos_plan_query", "nl
             "nlos_batch_create", "nlos_batch_launch", "nlos_batch_destroy", "nlos_plan_create_ex",
             "nlos_server_create", "nlos_server_preload", "nlos_server_submit", "nlos_server_wait",
             "nlos_server_stats", "nlos_server_destroy", "nlos_workspace_check", "nlos_selftest_bounded_wait",
+            "nlos_selftest_warp_wait",
             "nlos_max_image", "nlos_moe_mix", "nlos_coherence_merge", "nlos_dda",
             "nlos_bin_transient", "nlos_bin_phasors", "nlos_plan_band", "nlos_reconstruct_phasors",
             "nlos_reconstruct_host_many", "nlos_debug_fail_allocation", "nlos_selftest_umma",
@@ -106,6 +107,8 @@ def load_library(path: str = LIB_PATH):
     lib.nlos_workspace_check.restype = ctypes.c_int
     lib.nlos_selftest_bounded_wait.argtypes = [ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
     lib.nlos_selftest_bounded_wait.restype = ctypes.c_int
+    lib.nlos_selftest_warp_wait.argtypes = [ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
+    lib.nlos_selftest_warp_wait.restype = ctypes.c_int
     ll, fl = ctypes.c_longlong, ctypes.c_float
     lib.nlos_max_image.argtypes = [vp, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int, vp, vp]
     lib.nlos_moe_mix.argtypes = [vp, vp, ll, fl, fl, vp, vp]
