@@ -130,6 +130,19 @@ nlos_status_t nlos_plan_create(const nlos_plan_desc_t* desc, nlos_plan_t* out);
  * intermediate kept in L2; the inverse pair alone also for other nt in large
  * float32 plans). Same results up to rounding; for comparison and testing. */
 #define NLOS_PLAN_SEPARATE_AXES 2
+/* NLOS_PLAN_SMALL_WORKSPACE: the f-k stage structure with the smaller
+ * workspace where there is a choice. Large float32 zero-padded f-k plans take
+ * one temporal transform per stored pencil and one per wall point instead of
+ * three per stored pencil. If nt is no power of two that structure needs a
+ * larger workspace (it is chosen for workspaces above 32 MiB that grow by at
+ * most half). A plan that does not fit the device that way is created in the
+ * smaller form without the flag; a caller that supplies workspaces
+ * (nlos_reconstruct_ws, batches) under a limit of its own asks for it here.
+ * Same results up to rounding. 190 x 190 x 3002: 12.1 GiB and 8.0 ms, small
+ * 11.0 GiB and 15.0 ms. 16-bit plans whose nt is no power of two always have
+ * the smaller form and its three transforms (5.5 GiB, 15.1 ms).
+ */
+#define NLOS_PLAN_SMALL_WORKSPACE 4
 nlos_status_t nlos_plan_create_ex(const nlos_plan_desc_t* desc, int flags, nlos_plan_t* out);
 
 /*
@@ -523,7 +536,10 @@ nlos_status_t nlos_ffma_rate_launch(const float* params, float* sink, int blocks
  * device allocation that plan creation or host staging makes from now on
  * (k >= 1) fails as if the device were out of memory, and the call returns
  * NLOS_ERR_OUT_OF_MEMORY after releasing what it had allocated; k = 0
- * disables. Process-wide; not for production use. */
+ * disables. With k <= -1 the (-k)-th fails like that of a device that is out
+ * of memory: a plan that has a form with a smaller workspace
+ * (NLOS_PLAN_SMALL_WORKSPACE) is then created in that form. Process-wide; not
+ * for production use. */
 void nlos_debug_fail_allocation(int k);
 
 /*

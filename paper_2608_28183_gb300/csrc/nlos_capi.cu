@@ -208,7 +208,7 @@ struct nlos_plan_s {
   bool fused_inv = false;               // f-k lateral inverse transforms fused
   bool zlast = false;                   // f-k inverse temporal transform last (fk_zsplit.cuh)
   int zcols = 0;                        // columns (m or z) the f-k lateral inverses run over
-  bool injected = false;                // an allocation failed through the testing hook
+  bool injected = false;                // an allocation failed through the testing hook (k > 0)
   size_t ws_bytes = 0;
   void* ws = nullptr;
   // host-call staging
@@ -236,8 +236,10 @@ struct nlos_plan_s {
 
 namespace {
 
-// failure-path testing hook: the n-th plan allocation from now fails (0: off)
+// failure-path testing hook: the n-th plan allocation from now fails (0: off),
+// as an injected failure or (soft) as a device that is out of memory
 std::atomic<int> g_fail_alloc{0};
+std::atomic<bool> g_fail_soft{false};
 
 nlos_status_t dalloc(nlos_plan_s* p, void** ptr, size_t bytes, const char* what) {
   int k = g_fail_alloc.load();
@@ -245,7 +247,7 @@ nlos_status_t dalloc(nlos_plan_s* p, void** ptr, size_t bytes, const char* what)
   }
   if (k == 1) {
     *ptr = nullptr;
-    p->injected = true;
+    p->injected = !g_fail_soft.load();
     return fail(NLOS_ERR_OUT_OF_MEMORY, "%s: injected allocation failure", what);
   }
   cudaError_t e = cudaMalloc(ptr, bytes ? bytes : 16);
@@ -348,7 +350,8 @@ void fk_buffers(const nlos_plan_s* p, bool zlast, size_t* b0, size_t* b1, size_t
 //  * their buffers exceed 32 MiB: below that a volume takes a few launches of
 //    a few microseconds each and one stage more costs what it saves (and
 //    plans that fit nlos_reconstruct_noalloc's fixed scratch keep fitting);
-//  * their buffers grow by at most half (V has L/2 >= n columns).
+//  * their buffers grow by at most half (V has L/2 >= n columns);
+//  * the caller has not asked for the smaller workspace.
 // Measured: 190x190x3002 13.99 -> 8.12 ms, 96x80x300 269 -> 216 us. 16-bit plans
 // keep their order of roundings.
 void fk_structure(nlos_plan_s* p, int flags) {
@@ -358,7 +361,7 @@ void fk_structure(nlos_plan_s* p, int flags) {
   p->fused_inv = p->fused;
   p->zlast = p->fused && !fk_wide(p);
   p->zcols = p->n;
-  if (p->zlast || sep || d.pad_factor != 2 || p->storage != kF32 || (flags & kPlanSmallWorkspace)) return;
+  if (p->zlast || sep || d.pad_factor != 2 || p->storage != kF32 || (flags & NLOS_PLAN_SMALL_WORKSPACE)) return;
   size_t o[3], w[3];
   fk_buffers(p, false, &o[0], &o[1], &o[2]);
   fk_buffers(p, true, &w[0], &w[1], &w[2]);
@@ -368,6 +371,9 @@ void fk_structure(nlos_plan_s* p, int flags) {
   p->zcols = p->Lt / 2;
   p->fused_inv = fk_chain_inv_eligible(p->zcols, p->Lx, p->Ly);
 }
+
+// whether NLOS_PLAN_SMALL_WORKSPACE would give this plan a smaller workspace
+bool has_small_form(const nlos_plan_s* p) { return p->zlast && fk_wide(p); }
 
 nlos_status_t build_fk(nlos_plan_s* p) {
   const auto& d = p->d;
@@ -1514,10 +1520,10 @@ nlos_status_t nlos_plan_create_ex(const nlos_plan_desc_t* desc, int flags, nlos_
   if (st != NLOS_OK) {
     // device memory that does not hold this structure's buffers may hold the
     // smaller ones'
-    const bool again = st == NLOS_ERR_OUT_OF_MEMORY && !p->injected && p->zlast && fk_wide(p);
+    const bool again = st == NLOS_ERR_OUT_OF_MEMORY && !p->injected && has_small_form(p);
     for (void* v : p->allocs) cudaFree(v);
     delete p;
-    return again ? nlos_plan_create_ex(desc, flags | kPlanSmallWorkspace, out) : st;
+    return again ? nlos_plan_create_ex(desc, flags | NLOS_PLAN_SMALL_WORKSPACE, out) : st;
   }
   *out = p;
   return NLOS_OK;
@@ -2155,7 +2161,11 @@ nlos_status_t nlos_plan_destroy(nlos_plan_t p) {
   return NLOS_OK;
 }
 
-void nlos_debug_fail_allocation(int k) { g_fail_alloc.store(k > 0 ? k : 0); }
+void nlos_debug_fail_allocation(int k) {
+  g_fail_alloc.store(0);
+  g_fail_soft.store(k < 0);
+  g_fail_alloc.store(k < 0 ? -k : k);
+}
 
 const char* nlos_last_error(void) { return g_err.c_str(); }
 

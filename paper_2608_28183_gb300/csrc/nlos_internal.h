@@ -183,9 +183,6 @@ cudaError_t launch_fk_chain(const FkChainLaunch& l, int storage, cudaStream_t s)
 // the fused inverse alone: any a, b <= L / 2 (its copies are runs of blocked
 // columns), n columns a multiple of 16
 inline bool fk_chain_inv_eligible(int n, int Lx, int Ly) { return Lx == Ly && Lx >= 128 && Lx <= 1024 && n % 16 == 0; }
-// nlos_plan_create_ex flag for the library's own callers: the temporal stage
-// with the smaller workspace where there is a choice
-constexpr int kPlanSmallWorkspace = 1 << 8;
 // the pair: zero-padded f-k with Lx = Ly = L in [128, 1024] (at least one warp of
 // transforming threads per CTA), n a multiple of 16, and every TMA box row
 // count (a, b, L) at most 256 or a multiple of it

@@ -266,7 +266,7 @@ nlos_status_t acquire_plan(nlos_server_s* sv, const nlos_plan_desc_t& d, PlanEnt
   if (bytes + need > sv->budget) {
     // a structure with a smaller workspace may fit
     nlos_plan_destroy(p);
-    st = nlos_plan_create_ex(&d, NLOS_PLAN_NO_WORKSPACE | nlos::kPlanSmallWorkspace, &p);
+    st = nlos_plan_create_ex(&d, NLOS_PLAN_NO_WORKSPACE | NLOS_PLAN_SMALL_WORKSPACE, &p);
     if (st != NLOS_OK) return st;
     bytes = nlos::plan_resident_bytes(p);
     need = nlos::plan_workspace_bytes(p);

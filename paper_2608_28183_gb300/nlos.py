@@ -20,7 +20,7 @@ STATUS = {0: "OK", 1: "INVALID_ARG", 2: "OUT_OF_MEMORY", 3: "CUDA", 4: "UNSUPPOR
 METHODS = {"fk": NLOS_FK, "pf": NLOS_PHASOR_RSD, "phasor": NLOS_PHASOR_RSD, "pf_dense": NLOS_PHASOR_DENSE}
 STORAGES = {"f32": NLOS_F32, "f16": NLOS_F16, "bf16": NLOS_BF16}
 OUTPUTS = {"magnitude": 0, "complex": 1}
-PLAN_NO_WORKSPACE, PLAN_SEPARATE_AXES = 1, 2
+PLAN_NO_WORKSPACE, PLAN_SEPARATE_AXES, PLAN_SMALL_WORKSPACE = 1, 2, 4
 # bounds-checked debug build (NLOS_BOUNDS_CHECK=1): plans read their device
 # error word when closed and record nonzero codes here
 BOUNDS_CHECKED = os.environ.get("NLOS_BOUNDS_CHECK", "0") not in ("", "0")
@@ -207,14 +207,14 @@ class Plan:
 
     def __init__(self, nx: int, ny: int, nt: int, bin_width_s: float, wall_w_m: float, wall_h_m: float,
                  method: str = "fk", storage: str = "f32", pad_factor: int = 2, separate_axes: bool = False,
-                 **kw):
+                 small_workspace: bool = False, **kw):
         lib = load_library()
         d = make_desc(nx, ny, nt, bin_width_s, wall_w_m, wall_h_m, method, storage, pad_factor, **kw)
         self.desc = d
         self.method = method
         self.storage = storage
         h = ctypes.c_void_p()
-        flags = PLAN_SEPARATE_AXES if separate_axes else 0
+        flags = (PLAN_SEPARATE_AXES if separate_axes else 0) | (PLAN_SMALL_WORKSPACE if small_workspace else 0)
         self._own_ws = True
         _check(lib.nlos_plan_create_ex(ctypes.byref(d), flags, ctypes.byref(h)))
         self._h = h
