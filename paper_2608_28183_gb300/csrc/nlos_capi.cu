@@ -2181,6 +2181,7 @@ const char* nlos_version(void) { return "nlos-gb300 0.2 (sm_103a)"; }
 namespace nlos {
 size_t plan_workspace_bytes(const nlos_plan_s* p) { return p->ws_bytes; }
 size_t plan_resident_bytes(const nlos_plan_s* p) { return p->resident; }
+bool plan_has_small_form(const nlos_plan_s* p) { return has_small_form(p); }
 bool plan_profiling(const nlos_plan_s* p) { return p->prof_on; }
 nlos_status_t plan_run(nlos_plan_s* p, const void* H, void* vol, void* ws, cudaStream_t s) {
   return run_plan(p, H, vol, ws, s);

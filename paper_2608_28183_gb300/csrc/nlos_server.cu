@@ -47,6 +47,7 @@
 namespace nlos {
 size_t plan_workspace_bytes(const nlos_plan_s* p);
 size_t plan_resident_bytes(const nlos_plan_s* p);
+bool plan_has_small_form(const nlos_plan_s* p);
 nlos_status_t plan_run(nlos_plan_s* p, const void* H, void* vol, void* ws, cudaStream_t s);
 nlos_status_t set_error(nlos_status_t st, const char* msg);
 }  // namespace nlos
@@ -260,29 +261,26 @@ nlos_status_t acquire_plan(nlos_server_s* sv, const nlos_plan_desc_t& d, PlanEnt
     }
   }
   nlos_plan_t p = nullptr;
-  nlos_status_t st = nlos_plan_create_ex(&d, NLOS_PLAN_NO_WORKSPACE, &p);
-  if (st != NLOS_OK) return st;
-  size_t bytes = nlos::plan_resident_bytes(p), need = nlos::plan_workspace_bytes(p);
-  if (bytes + need > sv->budget) {
-    // a structure with a smaller workspace may fit
-    nlos_plan_destroy(p);
-    st = nlos_plan_create_ex(&d, NLOS_PLAN_NO_WORKSPACE | NLOS_PLAN_SMALL_WORKSPACE, &p);
+  size_t bytes = 0, need = 0;
+  for (int flags = NLOS_PLAN_NO_WORKSPACE;; flags |= NLOS_PLAN_SMALL_WORKSPACE) {
+    nlos_status_t st = nlos_plan_create_ex(&d, flags, &p);
     if (st != NLOS_OK) return st;
     bytes = nlos::plan_resident_bytes(p);
     need = nlos::plan_workspace_bytes(p);
-  }
-  if (bytes + need > sv->budget) {
+    // launch shapes picked once per description (the process-wide autotune
+    // cache): a resident plan serves every later request with the tuned shapes
+    const bool fits = bytes + need <= sv->budget;
+    st = fits ? nlos_plan_autotune(p, nullptr) : NLOS_ERR_OUT_OF_MEMORY;
+    if (st == NLOS_OK) break;
+    // a form of the plan with a smaller workspace may fit, if it has one
+    const bool again = st == NLOS_ERR_OUT_OF_MEMORY && nlos::plan_has_small_form(p);
     nlos_plan_destroy(p);
+    if (again) continue;
+    if (fits) return st;
     char msg[200];
     snprintf(msg, sizeof msg, "plan (%zu bytes) and workspace (%zu bytes) exceed the budget of %zu bytes", bytes,
              need, sv->budget);
     return nlos::set_error(NLOS_ERR_OUT_OF_MEMORY, msg);
-  }
-  // launch shapes picked once per description (the process-wide autotune
-  // cache): a resident plan serves every later request with the tuned shapes
-  if ((st = nlos_plan_autotune(p, nullptr)) != NLOS_OK) {
-    nlos_plan_destroy(p);
-    return st;
   }
   std::vector<nlos_plan_t> victims;
   {
