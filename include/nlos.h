@@ -232,7 +232,8 @@ nlos_status_t nlos_reconstruct_noalloc(nlos_plan_t plan, const void* transient, 
  * tensor-core, one-CTA-per-tile tensor-core and FP32-FMA forms) time the
  * whole reconstruction with each variant on a
  * scratch input (coordinate descent, CUDA events on `stream`) and keep the
- * fastest. Results are cached per plan shape for the process and, when the
+ * fastest. Results are cached per plan shape (capture, storage, stage
+ * structure, padding, output) for the process and, when the
  * environment variable NLOS_AUTOTUNE_CACHE names a file, in that JSON file
  * (read on first use, rewritten after tuning). Synchronous; allocates a
  * scratch transient and volume for the duration of the call. Variants

@@ -1794,11 +1794,19 @@ bool g_tune_loaded = false;
 
 std::string tune_key(const nlos_plan_s* p) {
   char buf[256];
-  // (the suffix keeps shapes tuned for another stage structure of the same
-  // capture apart)
-  snprintf(buf, sizeof buf, "m%d_s%d_%dx%dx%d_F%d_D%d%s", p->d.method, p->storage, p->a, p->b, p->n, p->F, p->D,
-           p->zlast && !(p->fused && !fk_wide(p)) ? (p->fused_inv ? "_zf" : "_z") : "");
-  return buf;
+  snprintf(buf, sizeof buf, "m%d_s%d_%dx%dx%d_F%d_D%d", p->d.method, p->storage, p->a, p->b, p->n, p->F, p->D);
+  // suffixes keep plans of the same capture apart whose stages differ: in
+  // structure, in transform lengths (unpadded f-k) or in the last stage's
+  // output. The padded magnitude plan of the default structure has none, so
+  // shapes saved for it stay valid.
+  std::string key = buf;
+  if (p->d.method == NLOS_FK) {
+    if (p->zlast && !(p->fused && !fk_wide(p))) key += p->fused_inv ? "_zf" : "_z";
+    if (!p->fused && fk_chain_eligible(p->a, p->b, p->n, p->Lx, p->Ly, p->d.pad_factor)) key += "_sep";
+    if (p->d.pad_factor == 1) key += "_p1";
+  }
+  if (p->d.output == NLOS_OUT_COMPLEX) key += "_cpx";
+  return key;
 }
 
 void tune_cache_load() {
