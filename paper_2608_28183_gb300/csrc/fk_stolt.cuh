@@ -19,7 +19,7 @@ __device__ __forceinline__ float2 fast_two_sum(float a, float b) {  // |a| >= |b
 }
 
 struct StoltCoord {
-  int k0, k1;
+  int k0;       // lower of the two samples around the source
   float alpha, jac;
   bool valid;
 };
@@ -46,7 +46,6 @@ __device__ __forceinline__ StoltCoord stolt_coord(float Ahi, float Alo, int m, i
   }
   c.valid = (k0 < n - 1) || (k0 == n - 1 && al == 0.f);
   c.k0 = k0;
-  c.k1 = min(k0 + 1, n - 1);
   c.alpha = al;
   c.jac = (float)m * rs;
   return c;
@@ -92,7 +91,6 @@ __device__ __forceinline__ StoltCoord stolt_coord_split(const StoltSplitA& a, fl
   const int k0 = __float_as_int(t0) + (__float_as_int(t1) - 2 * kFloorBits);
   c.valid = (k0 < n - 1) || (k0 == n - 1 && al == 0.f);
   c.k0 = k0;
-  c.k1 = k0 + 1;
   c.alpha = al;
   c.jac = fm * rs;
   return c;

@@ -83,8 +83,9 @@ struct FkInvCtx {
     if (m < 1) return;                                // m < L/2 (upper half is pruned)
     const StoltCoord c = stolt_coord(Ahi, Alo, m, n);
     if (!c.valid) return;
-    const float2 u0 = U[pad16(c.k0)], u1 = U[pad16(c.k1)];
-    const float2 w0 = U[pad16((L - c.k0) & (L - 1))], w1 = U[pad16((L - c.k1) & (L - 1))];
+    const int k1 = min(c.k0 + 1, n - 1);
+    const float2 u0 = U[pad16(c.k0)], u1 = U[pad16(k1)];
+    const float2 w0 = U[pad16((L - c.k0) & (L - 1))], w1 = U[pad16((L - k1) & (L - 1))];
     const float2 d = make_float2(fmaf(c.alpha, u1.x - u0.x, u0.x), fmaf(c.alpha, u1.y - u0.y, u0.y));
     const float2 e = make_float2(fmaf(c.alpha, w1.x - w0.x, w0.x), fmaf(c.alpha, w1.y - w0.y, w0.y));
     x[0] = cscale(d, c.jac);
