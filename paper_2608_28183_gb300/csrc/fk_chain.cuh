@@ -12,13 +12,13 @@
 //
 // Each item is one or two sub-tiles of IC = 8 columns. Sub-tiles stream
 // through two or three shared-memory slots: a producer warp takes the tickets, waits
-// for chunk counters and issues the TMA copy of the next sub-tile while the
-// other warps transform the current one (the scalar Stockham core of
-// nlos_fft.cuh with radix-32 passes, 32 values per thread, in place in the
-// slot).
+// for chunk counters and issues the copy of the next sub-tile (the transient: a
+// TMA box; the other three inputs: one bulk copy) while the other warps
+// transform the current one in place in the slot (the Stockham core of
+// nlos_fft.cuh; chain_e says where its passes are radix 32 and where 16).
 //
 // The intermediate of a chunk (about 8 MB at 256 x 256) is read within a few
-// microseconds of being written; once its TMA copies have landed, its L2
+// microseconds of being written; once a sub-tile's copy has landed, its L2
 // lines are dropped without write-back (discard.global.L2), so it never
 // reaches DRAM.
 //

@@ -1,8 +1,12 @@
 // Stolt source coordinate of the f-k temporal stage (Sec. 4.2, Alg. 1,
-// Listing 2) in float-float arithmetic: mu = sqrt(A + m^2) with A from
-// float64 per-plan tables split into (hi, lo) floats, m^2 exact, and one
-// Newton correction of the square root from an exact FMA residual. Plain
-// float would put the interpolation weight off by up to 6e-5 near m ~ 1000.
+// Listing 2): mu = sqrt(A + m^2) with A from float64 per-plan tables split
+// into (hi, lo) floats, m^2 exact, and one Newton correction of the square
+// root from an exact FMA residual. Plain float would put the interpolation
+// weight off by up to 6e-5 near m ~ 1000. Two forms: stolt_coord sums A + m^2
+// as float-float per m (the stages that keep their inverse transforms);
+// stolt_coord_split splits A once per pencil into an integer and a fraction
+// (the split stage of fk_zsplit.cuh). The errors of their weights agree: its
+// rounding to one float dominates both.
 #pragma once
 #include <cuda_runtime.h>
 

@@ -14,7 +14,7 @@
 //   3. inverse transform of the resampled Hermitian partner (-kx, -ky),
 //      conj(lerp(U[-k0], U[-k1])) m/mu, in place in U once every gather of it
 //      has been read.
-// Inverse transforms run as conj(DFT(conj(V))).
+// Inverse transforms turn the butterflies the other way (nlos_fft.cuh).
 //
 // Coordinate table: mu = sqrt(A + m^2) in float-float (stolt_coord) stored as
 // fixed point, k0 in the upper bits and the fraction alpha in the lower

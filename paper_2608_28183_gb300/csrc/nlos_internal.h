@@ -168,7 +168,7 @@ struct FkChainParams {
   const float* st_dev_scale;   // inverse: optional device scalar multiplying the output
   int* sync;                   // [1 + nchunks] ints, zero at launch: ticket, finished first-transform items per chunk
   int* err;                    // device error word
-  int discard;                 // drop consumed lines of `mid` from L2 (float32 storage)
+  int discard;                 // drop the whole lines of consumed runs of `mid` from L2
   long long in_n, mid_n, out_n;  // element extents (bounds-checked build; 0: unchecked)
 };
 struct FkChainLaunch {
@@ -176,7 +176,7 @@ struct FkChainLaunch {
   bool after;                  // launched after another kernel of the same call (nlos_launch.cuh)
   CUtensorMap map;             // forward: TMA map of the transient
   int fwd;                     // 1 forward, 0 inverse
-  int store_mode;              // inverse: kStoreAbs2 or kStoreCpx32
+  int store_mode;              // inverse: kStoreAbs2, kStoreCpx32 or kStoreCpx (the storage type)
   int nslot;                   // shared-memory slots per CTA (2 or 3; 2 at L = 1024)
 };
 cudaError_t launch_fk_chain(const FkChainLaunch& l, int storage, cudaStream_t s);

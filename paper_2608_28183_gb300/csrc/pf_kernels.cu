@@ -653,8 +653,8 @@ template <class T> __device__ __forceinline__ T tree_sum256(const T* r, int lane
   return x;
 }
 
-// The last CTA to finish (a counter in the partials' array, reset by that
-// CTA) sums the partials in index order and writes the scale, its inverse
+// The last CTA to finish (a counter in the partials' array, cleared by the host
+// ahead of the launch) sums the partials in index order and writes the scale, its inverse
 // and the inverse square: the result does not depend on CTA timing.
 // The vector's read is at the memory's rate; what is left is the chain after
 // it, so the last loads of a thread and the partials go out together and the
